@@ -153,12 +153,17 @@ typedef struct {
                             finished blocks leave. */
   int32_t use_graph;     /* 1: capture the launch sequence once per call shape, then replay */
   int32_t ef_max;        /* bound on ef' over the batch when per-query ef is given; 0 => 512 */
-  int32_t query_threads; /* threads per query: 32 = one warp per query (4 queries per
-                            block), 128 = one block per query; a launch that does not fit
-                            in shared memory fails with UHNSW_ECAPACITY.  0 => the
-                            configuration uhnsw_autotune chose for this beam / k bucket,
-                            else 32; then a beam bucket whose warp-kernel layout does not
-                            fit runs the block kernel. */
+  int32_t query_threads; /* 32 = one warp per query (4 queries per block), 128 = one block per
+                            query (2, 4 or 8 warps sum its rows and one keeps its beam: the
+                            most with which all queries of the launch are resident at once,
+                            else 2); a launch that does not fit in shared memory fails with
+                            UHNSW_ECAPACITY.  0 => the configuration uhnsw_autotune chose for
+                            this beam / k bucket; else, with team_lanes and stage_bytes 0 too,
+                            a block per query where all queries are resident at once and for
+                            wide rows; else one warp per query, and for a beam bucket whose
+                            warp layout does not fit a block per query.  Both forms sum every
+                            row in the same order where they use one team shape, and return
+                            the same ids and distances. */
   int32_t* stats;        /* device [nq][UHNSW_NSTATS] int32, or NULL */
   int32_t stage_bytes;   /* warp kernel: shared memory per query for the FP32 rows being
                             verified (a multiple of 4 rows); 0 => as many rows as fit in
@@ -181,7 +186,8 @@ typedef struct {
                                   0.92, negative => stop after the first batch) */
   int32_t hash_bits;     /* visited table of 1 << hash_bits slots per query; 0 => the
                             smallest power of two >= 4 (ef' + search_width * M0), at least
-                            2^9.  Allowed: from the smallest power of two >= 2 (ef' +
+                            2^9 (a block per query: up to 2^14 where the shared memory of the
+                            resident queries allows).  Allowed: from the smallest power of two >= 2 (ef' +
                             search_width * M0) up to 2^15 (else UHNSW_EINVAL).  The size
                             does not change any result (a table past half full is cleared
                             and refilled with the beam, which cannot change the beam); a
@@ -191,7 +197,7 @@ typedef struct {
                             groups accumulated between two tests of a candidate's partial
                             sum against the running k-th best sum, 1..16; 0 => 2 in
                             uhnsw_search, 1 in uhnsw_verify (the block-per-query kernel
-                            tests after every group).  Every lane
+                            tests after every four).  Every lane
                             accumulates its elements in the same order whatever the
                             value, so sums and results do not depend on it; it trades
                             drop-test work for candidates summed further before they are

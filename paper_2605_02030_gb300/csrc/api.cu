@@ -14,6 +14,7 @@
 #include <new>
 #include <vector>
 
+#include "coop_kernels.cuh"
 #include "launch.h"
 #include "uhnsw.h"
 #include "uhnsw_internal.h"
@@ -252,7 +253,7 @@ GraphDev to_dev(const DevGraph& g) {
   return r;
 }
 
-constexpr int kBlock = 128;
+constexpr int kBlock = 128;  // uhnsw_search_opts.query_threads of the block-per-query form
 
 // The p of a base metric code 1-4 (uhnsw_base_metric).
 float base_metric_p(int32_t m) {
@@ -389,15 +390,14 @@ namespace {
 
 struct Launch {
   QueryArgs a;
-  bool warp;     // warp-per-query kernel, else block-per-query
+  int coop = 0;  // cooperative kernel with this many distance warps per query (0: warp kernel)
+  WarpShape shape;
   size_t smem;
   int grid;
 };
 
 struct Prepared {
   QueryArgs a;
-  TeamShape shape;    // block-per-query kernel
-  WarpShape wshape;   // warp-per-query kernel
   bool persistent;
   // persistent search: the queue is ordered by (beam bucket, route); with
   // per-query ef, one launch per beam bucket, largest first, each sized for
@@ -511,7 +511,7 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
     return fail(UHNSW_EINVAL, "uhnsw_search: beam %d exceeds %d", ef_cap, UHNSW_MAX_EF);
   // query_threads given by the caller is binding; otherwise (0, or the
   // autotuned choice) a beam bucket whose warp-kernel layout does not fit in
-  // shared memory runs the block kernel instead
+  // shared memory runs the cooperative kernel instead
   const bool forced = opts.query_threads != 0;
   if (opts.query_threads == 0) {
     // the autotuned configuration of this bucket, if any
@@ -541,9 +541,8 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
     return fail(UHNSW_EINVAL, "uhnsw_search: hash_bits=%d below the minimum %d for beam %d",
                 opts.hash_bits, next_pow2_bits(2ll * (ef_cap + width * deg0)), ef_cap);
   const int chunks = idx->d_pad / (idx->tdtype == UHNSW_F32 ? 4 : 8);
-  TeamShape sh{0, 0};
-  WarpShape wsh{0, 0, 0};
-  const bool have_block = pick_shape(idx->tdtype, chunks, &sh);
+  WarpShape bsh{0, 0, 0}, wsh{0, 0, 0};
+  const bool have_block = pick_block_shape(idx->tdtype, chunks, &bsh);
   const bool few = nq < (int64_t)idx->num_sms * WarpMinBlocks<float>::value * kWarpsPerBlock;
   const bool have_warp = pick_warp_shape(idx->tdtype, chunks, opts.team_lanes, few, &wsh);
   if (want_warp ? !have_warp : !have_block)
@@ -595,8 +594,6 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
   a.trav_exact = idx->trav_exact ? 1 : 0;
   a.queue_head = nullptr;  // set below for a persistent search
   a.sb = 0;
-  P->shape = sh;
-  P->wshape = wsh;
   P->persistent = opts.persistent != 0;
   if (opts.kernel_events) {
     const cudaEvent_t* ev = static_cast<const cudaEvent_t*>(opts.kernel_events);
@@ -605,39 +602,89 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
     P->events[1] = ev[1];
   }
 
+  // The cooperative kernel with the most distance warps that keep all queries
+  // resident at once: a launch that small is bound by each query's own chain of
+  // steps, and more warps shorten it (1M x 128 FP16, ef 64, one query: 8 warps
+  // 85 us, 4 warps 99, 2 warps 104, the warp kernel 194).  Queries that cannot
+  // all be resident: `fallback` warps, or no (false) for 0.
+  auto describe_coop = [&](int bound, const WarpShape& sh, int fallback, Launch* Lo) -> bool {
+    const int64_t per_sm = (nq + idx->num_sms - 1) / idx->num_sms;
+    for (int i = kCoopForms - 1; i >= -1; --i) {
+      const int nw = i >= 0 ? kCoopWarps[i] : fallback;
+      if (nw == 0) return false;
+      const int cmax = (std::max(width * deg0, deg) + nw - 1) / nw * nw;
+      const int ext = sh.team * sh.cpl * (idx->tdtype == UHNSW_F32 ? 4 : 8);
+      int hb = Lo->a.hash_bits;
+      size_t smem = CoopLayout(ext, bound, hb, cmax, k_max, nw + 1).total;
+      const int occ = csearch_occupancy(idx->tdtype, nw, sh, smem);
+      if (occ < 1 || (i >= 0 && occ < per_sm)) continue;
+      // a larger visited table re-evaluates fewer nodes; it takes the shared
+      // memory that the resident queries leave
+      while (opts.hash_bits == 0 && hb < 14) {
+        const size_t more = CoopLayout(ext, bound, hb + 1, cmax, k_max, nw + 1).total;
+        if (csearch_occupancy(idx->tdtype, nw, sh, more) < std::min<int64_t>(per_sm, occ)) break;
+        ++hb;
+        smem = more;
+      }
+      Lo->coop = nw;
+      Lo->shape = sh;
+      Lo->smem = smem;
+      Lo->a.hash_bits = hb;
+      Lo->a.cmax = cmax;
+      Lo->grid = (int)std::min<int64_t>(nq, P->persistent ? (int64_t)occ * idx->num_sms : nq);
+      return true;
+    }
+    return false;
+  };
+
+  // Distance warps per query of a launch whose queries are not all resident (0:
+  // the warp kernel).  Measured against the warp kernel, 2 warps per query:
+  //   rows above 64 chunks (960 BF16, 1,023 FP32): 0.98 to 1.99 times its
+  //     speed at 1,500 to 10,000 queries, ef 52 to 300;
+  //   33 to 64 chunks (500 FP16, 200 and 500 FP32): 1.04 to 2.4 at ef 300;
+  //     at ef 52 and 64, 1.15 to 1.75 up to 2,500 queries, 0.67 to 1.28 above;
+  //   narrower rows: 0.7 to 1.4 at 1,500 queries, 0.6 to 0.9 at 10,000.
+  auto coop_anyway = [&](const WarpShape& sh, int bound) -> int {
+    const int row = sh.team * sh.cpl;
+    if (row > 64) return 2;
+    if (row > 32 && (bound > 128 || nq <= 20 * (int64_t)idx->num_sms)) return 2;
+    return 0;
+  };
+
   // One launch description for a beam bound: kernel kind, layout, grid.
   auto describe = [&](int bound, Launch* Lo) -> int {
     Lo->a = a;
     Lo->a.ef_cap = bound;
     Lo->a.hash_bits = visited_bits(opts.hash_bits, bound, width, deg0);
-    bool w = want_warp;
-    for (int attempt = 0; attempt < 2; ++attempt) {
-      const int cmax = std::max({width * deg0, deg, w ? 4 : kBlock / 8});
+    if (want_warp) {
+      // the caller's (or the autotuner's) kernel, team or staging is kept
+      if (opts.query_threads == 0 && opts.team_lanes == 0 && opts.stage_bytes == 0 &&
+          describe_coop(bound, wsh, coop_anyway(wsh, bound), Lo))
+        return UHNSW_OK;
+      const int cmax = std::max({width * deg0, deg, 4});
       const int sv = sv_asked > 0 ? sv_asked
                                   : std::min(16, std::max(4, (((1 << Lo->a.hash_bits) * 4) / vrow) & ~3));
-      const int stage = w ? sv * vrow : 0;
-      const SmemLayout Lw(idx->d_pad, bound, Lo->a.hash_bits, cmax, k_max, 0, stage);
-      const size_t smem = w ? (size_t)Lw.total * kWarpsPerBlock : (size_t)Lw.total;
+      const SmemLayout Lw(idx->d_pad, bound, Lo->a.hash_bits, cmax, k_max, 0, sv * vrow);
+      const size_t smem = (size_t)Lw.total * kWarpsPerBlock;
       if (smem <= kSmemMax) {
-        Lo->warp = w;
+        Lo->shape = wsh;
         Lo->smem = smem;
         Lo->a.cmax = cmax;
-        Lo->a.stage_bytes = stage;
-        Lo->a.sv = w ? sv : 0;
-        const int64_t per_block = w ? kWarpsPerBlock : 1;
-        Lo->grid = (int)((nq + per_block - 1) / per_block);
+        Lo->a.stage_bytes = sv * vrow;
+        Lo->a.sv = sv;
+        Lo->grid = (int)((nq + kWarpsPerBlock - 1) / kWarpsPerBlock);
         if (P->persistent) {
-          const int occ = w ? wsearch_occupancy(idx->tdtype, wsh, smem)
-                            : search_occupancy(idx->tdtype, sh, kBlock, smem);
+          const int occ = wsearch_occupancy(idx->tdtype, wsh, smem);
           if (occ < 1) return fail(UHNSW_ECUDA, "uhnsw_search: kernel does not fit (smem %zu)", smem);
           Lo->grid = (int)std::min<int64_t>(Lo->grid, (int64_t)occ * idx->num_sms);
         }
         return UHNSW_OK;
       }
-      if (!w || forced || !have_block)
+      if (forced || !have_block)
         return fail(UHNSW_ECAPACITY, "uhnsw_search: %zu bytes of shared memory per block", smem);
-      w = false;  // the block kernel holds one query per block
     }
+    // the block-per-query form: one query per block
+    if (describe_coop(bound, bsh, 2, Lo)) return UHNSW_OK;
     return fail(UHNSW_ECAPACITY, "uhnsw_search: no launch fits");
   };
 
@@ -690,8 +737,8 @@ int enqueue_search(uhnsw_index* idx, const Prepared& P, cudaStream_t st) {
     if (e != cudaSuccess) return cuda_fail(e, "uhnsw_search: kernel_events[0]");
   }
   for (const Launch& L : P.launches) {
-    e = L.warp ? launch_wsearch(idx->tdtype, P.wshape, L.a, L.grid, L.smem, st)
-               : launch_search(idx->tdtype, P.shape, L.a, L.grid, kBlock, L.smem, st);
+    e = L.coop ? launch_csearch(idx->tdtype, L.coop, L.shape, L.a, L.grid, L.smem, st)
+               : launch_wsearch(idx->tdtype, L.shape, L.a, L.grid, L.smem, st);
     if (e != cudaSuccess) return cuda_fail(e, "uhnsw_search: launch");
   }
   if (P.events[1]) {
@@ -1133,7 +1180,7 @@ extern "C" int uhnsw_autotune(uhnsw_index* idx, const float* q, const float* p, 
           cands.push_back(c);
         }
   }
-  for (int hb : hbs) {  // (the block kernel tests after every group: no interval to try)
+  for (int hb : hbs) {  // (the block-per-query form has a fixed drop-test interval)
     uhnsw_search_opts c = b;
     c.query_threads = kBlock;
     c.team_lanes = 0;

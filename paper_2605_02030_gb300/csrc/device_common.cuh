@@ -25,14 +25,6 @@ template <> struct Elems16<float> { static constexpr int n = 4; };
 template <> struct Elems16<__half> { static constexpr int n = 8; };
 template <> struct Elems16<__nv_bfloat16> { static constexpr int n = 8; };
 
-__device__ __forceinline__ uint4 ldg16(const void* p) {
-  uint4 r;
-  asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
-               : "l"(p));
-  return r;
-}
-
 template <typename T>
 __device__ __forceinline__ void unpack16(const uint4& v, float* out);
 
@@ -165,48 +157,6 @@ __device__ __forceinline__ int lower_bound_pair(const float* d, const uint32_t* 
     else hi = mid;
   }
   return lo;
-}
-
-// Block-wide merge of m unsorted new entries (nd, ni) into the ascending list
-// (ld, li) of n entries, keeping the first `cap` of the union in (od, oi).
-// Ids carry a flag in bit 31 that is preserved; flag-free ids are unique.
-// sd/si is scratch for m entries.  Returns the new length; *first_flagless
-// (if non-null) receives the smallest output position whose flag is clear
-// (INT_MAX if none).  Must be called by every thread of the block; ends with
-// a barrier.
-__device__ __forceinline__ int block_merge(const float* ld, const uint32_t* li, int n,
-                                           const float* nd, const uint32_t* ni, int m, float* sd,
-                                           uint32_t* si, float* od, uint32_t* oi, int cap,
-                                           int* first_flagless) {
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    float x = nd[i];
-    int32_t xi = (int32_t)(ni[i] & kIdMask);
-    int r = 0;
-    for (int j = 0; j < m; ++j) r += pair_lt(nd[j], (int32_t)(ni[j] & kIdMask), x, xi);
-    r = (int)chk_idx(r, m, 8, nullptr);
-    sd[r] = x;
-    si[r] = ni[i];
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    int pos = lower_bound_pair(ld, li, n, sd[i], (int32_t)(si[i] & kIdMask)) + i;
-    if (pos < cap) {
-      od[pos] = sd[i];
-      oi[pos] = si[i];
-      if (first_flagless && !(si[i] & kExpanded)) atomicMin(first_flagless, pos);
-    }
-  }
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    int pos = lower_bound_pair(sd, si, m, ld[j], (int32_t)(li[j] & kIdMask)) + j;
-    if (pos < cap) {
-      od[pos] = ld[j];
-      oi[pos] = li[j];
-      if (first_flagless && !(li[j] & kExpanded)) atomicMin(first_flagless, pos);
-    }
-  }
-  __syncthreads();
-  int total = n + m;
-  return total < cap ? total : cap;
 }
 
 // Two FP32 lanes in one 64-bit register: Blackwell's paired FP32 instructions

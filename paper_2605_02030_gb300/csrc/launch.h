@@ -10,15 +10,6 @@
 
 namespace uhnsw_dev {
 
-// Team shape of the traversal distance: TEAM lanes per row, CPL 16-byte chunks
-// per lane; the first shape whose TEAM * CPL covers the row is used.
-struct TeamShape {
-  int team, cpl;
-};
-
-// Returns false if no compiled shape covers rows of `chunks` 16-byte chunks.
-bool pick_shape(uhnsw_dtype dt, int chunks, TeamShape* out);
-
 // Warp-per-query kernel: TEAM lanes per row, CPL 16-byte chunks per lane,
 // U rows per team loaded per round; 4 warps (queries) per block.
 struct WarpShape {
@@ -35,13 +26,19 @@ cudaError_t launch_wsearch(uhnsw_dtype dt, WarpShape sh, const QueryArgs& a, int
                            size_t smem, cudaStream_t st);
 int wsearch_occupancy(uhnsw_dtype dt, WarpShape sh, size_t smem);
 
-// Launch the fused search kernel: one block per query (grid = nq) or, with
-// a.queue_head set, `grid` persistent blocks.
-cudaError_t launch_search(uhnsw_dtype dt, TeamShape sh, const QueryArgs& a, int grid, int block,
-                          size_t smem, cudaStream_t st);
-
-// Resident blocks per SM of the search kernel for this shape and smem size.
-int search_occupancy(uhnsw_dtype dt, TeamShape sh, int block, size_t smem);
+// Cooperative kernel (coop_kernels.cuh): one query per block, kCoopWarps[i]
+// distance warps and one merge warp.
+constexpr int kCoopForms = 3;
+constexpr int kCoopWarps[kCoopForms] = {2, 4, 8};
+// The block-per-query form's team shape where the caller asks for that form:
+// the first compiled shape that covers rows of `chunks` 16-byte chunks (false:
+// none does).
+bool pick_block_shape(uhnsw_dtype dt, int chunks, WarpShape* out);
+cudaError_t launch_csearch(uhnsw_dtype dt, int warps, WarpShape sh, const QueryArgs& a, int grid,
+                           size_t smem, cudaStream_t st);
+// Resident blocks per SM with `smem` bytes of shared memory per block (0: does
+// not fit).
+int csearch_occupancy(uhnsw_dtype dt, int warps, WarpShape sh, size_t smem);
 
 // Verification only, one warp per query (4 per block).
 cudaError_t launch_wverify(const QueryArgs& a, cudaStream_t st);
@@ -77,24 +74,42 @@ cudaError_t launch_exact(const float* base, int64_t n, int d, int d_pad, const f
                          const float* p, int64_t nq, int k, int nslices, float* part_d,
                          int32_t* part_i, int64_t* out_ids, float* out_dist, cudaStream_t st);
 
-// per-storage-type entry points (defined in search_<type>.cu)
-cudaError_t launch_search_f32(TeamShape sh, const QueryArgs& a, int grid, int block, size_t smem,
-                              cudaStream_t st);
-cudaError_t launch_search_f16(TeamShape sh, const QueryArgs& a, int grid, int block, size_t smem,
-                              cudaStream_t st);
-cudaError_t launch_search_bf16(TeamShape sh, const QueryArgs& a, int grid, int block, size_t smem,
-                               cudaStream_t st);
-int occupancy_f32(TeamShape sh, int block, size_t smem);
+// per-storage-type entry points (defined in wsearch_<type>.cu and csearch_<type>_w<warps>.cu)
 cudaError_t launch_wsearch_f32(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
                                cudaStream_t st);
+int wocc_f32(WarpShape sh, size_t smem);
+cudaError_t launch_csearch_f32_w2(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
+                                 cudaStream_t st);
+int csearch_regs_f32_w2(WarpShape sh);
+cudaError_t launch_csearch_f32_w4(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
+                                 cudaStream_t st);
+int csearch_regs_f32_w4(WarpShape sh);
+cudaError_t launch_csearch_f32_w8(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
+                                 cudaStream_t st);
+int csearch_regs_f32_w8(WarpShape sh);
 cudaError_t launch_wsearch_f16(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
                                cudaStream_t st);
-cudaError_t launch_wsearch_bf16(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
-                                cudaStream_t st);
-int wocc_f32(WarpShape sh, size_t smem);
 int wocc_f16(WarpShape sh, size_t smem);
+cudaError_t launch_csearch_f16_w2(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
+                                 cudaStream_t st);
+int csearch_regs_f16_w2(WarpShape sh);
+cudaError_t launch_csearch_f16_w4(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
+                                 cudaStream_t st);
+int csearch_regs_f16_w4(WarpShape sh);
+cudaError_t launch_csearch_f16_w8(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
+                                 cudaStream_t st);
+int csearch_regs_f16_w8(WarpShape sh);
+cudaError_t launch_wsearch_bf16(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
+                               cudaStream_t st);
 int wocc_bf16(WarpShape sh, size_t smem);
-int occupancy_f16(TeamShape sh, int block, size_t smem);
-int occupancy_bf16(TeamShape sh, int block, size_t smem);
+cudaError_t launch_csearch_bf16_w2(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
+                                 cudaStream_t st);
+int csearch_regs_bf16_w2(WarpShape sh);
+cudaError_t launch_csearch_bf16_w4(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
+                                 cudaStream_t st);
+int csearch_regs_bf16_w4(WarpShape sh);
+cudaError_t launch_csearch_bf16_w8(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
+                                 cudaStream_t st);
+int csearch_regs_bf16_w8(WarpShape sh);
 
 }  // namespace uhnsw_dev

@@ -58,12 +58,13 @@ cudaError_t launch_convert(const float* src, void* dst, uhnsw_dtype dt, int64_t 
   return cudaGetLastError();
 }
 
-bool pick_shape(uhnsw_dtype dt, int chunks, TeamShape* out) {
-  static const TeamShape f32[] = {{8, 1}, {16, 2}, {32, 2}, {32, 4}, {32, 8}, {32, 16}};
-  static const TeamShape f16[] = {{8, 1}, {16, 1}, {32, 1}, {32, 2}, {32, 4}, {32, 8}};
-  const TeamShape* list = dt == UHNSW_F32 ? f32 : f16;
-  const int cnt = 6;
-  for (int i = 0; i < cnt; ++i)
+bool pick_block_shape(uhnsw_dtype dt, int chunks, WarpShape* out) {
+  static const WarpShape f32[] = {{8, 1, 0},  {16, 2, 0}, {32, 2, 0},
+                                  {32, 4, 0}, {32, 8, 0}, {32, 16, 0}};
+  static const WarpShape f16[] = {{8, 1, 0},  {16, 1, 0}, {32, 1, 0},
+                                  {32, 2, 0}, {32, 4, 0}, {32, 8, 0}};
+  const WarpShape* list = dt == UHNSW_F32 ? f32 : f16;
+  for (int i = 0; i < 6; ++i)
     if (list[i].team * list[i].cpl >= chunks) {
       *out = list[i];
       return true;
@@ -205,22 +206,32 @@ int wsearch_occupancy(uhnsw_dtype dt, WarpShape sh, size_t smem) {
   return 0;
 }
 
-cudaError_t launch_search(uhnsw_dtype dt, TeamShape sh, const QueryArgs& a, int grid, int block,
-                          size_t smem, cudaStream_t st) {
-  switch (dt) {
-    case UHNSW_F32: return launch_search_f32(sh, a, grid, block, smem, st);
-    case UHNSW_F16: return launch_search_f16(sh, a, grid, block, smem, st);
-    case UHNSW_BF16: return launch_search_bf16(sh, a, grid, block, smem, st);
-  }
+cudaError_t launch_csearch(uhnsw_dtype dt, int warps, WarpShape sh, const QueryArgs& a, int grid,
+                           size_t smem, cudaStream_t st) {
+  using Fn = cudaError_t (*)(WarpShape, const QueryArgs&, int, size_t, cudaStream_t);
+  static const Fn fn[3][kCoopForms] = {
+      {launch_csearch_f32_w2, launch_csearch_f32_w4, launch_csearch_f32_w8},
+      {launch_csearch_f16_w2, launch_csearch_f16_w4, launch_csearch_f16_w8},
+      {launch_csearch_bf16_w2, launch_csearch_bf16_w4, launch_csearch_bf16_w8}};
+  for (int i = 0; i < kCoopForms; ++i)
+    if (kCoopWarps[i] == warps) return fn[(int)dt][i](sh, a, grid, smem, st);
   return cudaErrorInvalidValue;
 }
 
-int search_occupancy(uhnsw_dtype dt, TeamShape sh, int block, size_t smem) {
-  switch (dt) {
-    case UHNSW_F32: return occupancy_f32(sh, block, smem);
-    case UHNSW_F16: return occupancy_f16(sh, block, smem);
-    case UHNSW_BF16: return occupancy_bf16(sh, block, smem);
-  }
+int csearch_occupancy(uhnsw_dtype dt, int warps, WarpShape sh, size_t smem) {
+  using Fn = int (*)(WarpShape);
+  static const Fn fn[3][kCoopForms] = {
+      {csearch_regs_f32_w2, csearch_regs_f32_w4, csearch_regs_f32_w8},
+      {csearch_regs_f16_w2, csearch_regs_f16_w4, csearch_regs_f16_w8},
+      {csearch_regs_bf16_w2, csearch_regs_bf16_w4, csearch_regs_bf16_w8}};
+  constexpr size_t kSmSmem = 228 * 1024, kBlockReserve = 1024, kBlockMax = 227 * 1024;
+  if (smem > kBlockMax) return 0;
+  for (int i = 0; i < kCoopForms; ++i)
+    if (kCoopWarps[i] == warps) {
+      const int by_smem = (int)(kSmSmem / (smem + kBlockReserve));
+      const int by_regs = fn[(int)dt][i](sh);
+      return by_smem < by_regs ? by_smem : by_regs;
+    }
   return 0;
 }
 

@@ -1,5 +1,5 @@
-// Warp-per-query form of the query kernel (same algorithm and result as
-// uhnsw_search_kernel in query_kernels.cuh, Section 3.1 / Algorithm 1).
+// Warp-per-query form of the query kernel (Section 3.1, Algorithm 1; the
+// algorithm and why its search is HNSW's are set out in query_kernels.cuh).
 //
 // Each warp owns one query at a time and a private slice of the block's
 // shared memory (query vector, the two ping-pong lists of W, the visited
@@ -18,7 +18,7 @@
 // The search order is HNSW's (one expansion per step when width == 1), the
 // merge keeps the best ef' of W and the new candidates by (distance, id), and
 // the verification uses the same 8-lane teams and 32-dimension groups as the
-// block kernel, so both kernels return identical ids and distances.
+// cooperative kernel, so both kernels return identical ids and distances.
 #pragma once
 
 #include "query_kernels.cuh"
@@ -31,7 +31,7 @@ __device__ __forceinline__ int warp_min_int(int v) {
   return v;
 }
 
-// Warp version of block_merge: m unsorted new entries (nd, ni) into the
+// Merge by one warp: m unsorted new entries (nd, ni) into the
 // ascending (ld, li) of n entries, first `cap` of the union into (od, oi).
 // Returns the new length; *first receives the smallest output position of an
 // entry without the flag bit (INT_MAX if none), identical in every lane.
@@ -309,8 +309,12 @@ __device__ __forceinline__ float add_terms4(float acc, const float4& x, const fl
   acc += pow_term<PM>(fabsf(x.w - q.w), p);
   return acc;
 }
-// L_p sum of a staged FP32 row (shared memory) by a team of 8 lanes, with the
-// same grouping and drop test as lp_sum_team.  The p form `pm` selects the
+// L_p sum of a staged FP32 row (shared memory) by a team of 8 lanes: 4
+// consecutive dimensions per lane, 32 per group.  Every vgroups groups the
+// team's partial sum is compared with thr: once it is larger the candidate is
+// dropped (returns false).  Partial sums of non-negative FP32 terms never
+// decrease (the butterfly sum is monotone in every argument), so a dropped
+// candidate cannot belong to the K smallest.  The p form `pm` selects the
 // term code per 32-dimension group (a uniform branch), so that the
 // verification exists once in the kernel and not once per p form.
 __device__ __forceinline__ bool lp_sum_team_staged(const float* srow, int d, int d_pad,
@@ -808,8 +812,8 @@ __device__ void warp_query(const QueryArgs& a, int64_t qi, unsigned char* ws, co
 // 32-dimension groups at a time into registers, all loads of a block issued
 // before any arithmetic, so that the SFU work of one candidate overlaps the
 // other's reductions and the next block's loads.  Every lane sums the same
-// elements in the same order as lp_sum_team (element j = 32 g + 4 lane + e),
-// so the sums are bit-identical to the block kernel's.
+// elements in the same order as lp_sum_team_staged (element j = 32 g + 4 lane
+// + e), so the sums are bit-identical to the searches'.
 
 // Shared-memory carve-up of one warp of the verification-only kernel.
 struct WVerifyLayout {
