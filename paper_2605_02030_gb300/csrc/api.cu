@@ -970,10 +970,8 @@ extern "C" int uhnsw_exact(uhnsw_index* idx, const float* q, const float* p, int
     if (e != cudaSuccess) return cuda_fail(e, "uhnsw_exact: workspace");
     idx->exact_ws_bytes = need;
   }
-  float* pd = (float*)idx->exact_ws;
-  int32_t* pi = (int32_t*)((char*)idx->exact_ws + (size_t)ns * nq * k * 4);
-  cudaError_t e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, p, nq, k, ns, pd, pi,
-                               out_ids, out_dist, (cudaStream_t)stream);
+  cudaError_t e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, p, nq, k, ns,
+                               idx->exact_ws, out_ids, out_dist, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "uhnsw_exact: launch");
   return UHNSW_OK;
 }
@@ -1008,16 +1006,14 @@ extern "C" int uhnsw_idealized_recall(uhnsw_index* idx, const float* q, const fl
   int64_t* it = (int64_t*)s; s += al(b_it);
   float* dt = (float*)s; s += al(b_dt);
   float* pb = (float*)s; s += al(b_pb);
-  float* pd = (float*)s;
+  void* ws = s;
   cudaStream_t st = (cudaStream_t)stream;
   const float gp0 = idx->gp[0], gp1 = idx->gp[1];
   // exact L_p top-K, exact base-metric top-t_max, then the curves
-  e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, p, nq, K, ns, pd,
-                   (int32_t*)((char*)pd + (size_t)ns * nq * K * 4), ik, dk, st);
+  e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, p, nq, K, ns, ws, ik, dk, st);
   if (e == cudaSuccess) e = launch_base_p(p, nq, gp0, gp1, cut, pb, st);
   if (e == cudaSuccess)
-    e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, pb, nq, t_max, ns, pd,
-                     (int32_t*)((char*)pd + (size_t)ns * nq * t_max * 4), it, dt, st);
+    e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, pb, nq, t_max, ns, ws, it, dt, st);
   if (e == cudaSuccess) e = launch_recall_curve(ik, it, nq, K, t_max, counts, st);
   cudaError_t e2 = cudaStreamSynchronize(st);
   cudaFree(buf);
@@ -1103,9 +1099,7 @@ extern "C" int uhnsw_exact_static(uhnsw_index* idx, const float* q, const float*
   int ns = exact_workspace_slices(idx->n, nq, k, idx->num_sms);
   const int64_t fit = (int64_t)UHNSW_EXACT_STATIC_BYTES / per_slice;
   if (ns > fit) ns = (int)fit;
-  float* pd = (float*)base;
-  int32_t* pi = (int32_t*)((char*)base + (size_t)ns * nq * k * 4);
-  e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, p, nq, k, ns, pd, pi, out_ids,
+  e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, p, nq, k, ns, base, out_ids,
                    out_dist, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "uhnsw_exact_static: launch");
   return UHNSW_OK;

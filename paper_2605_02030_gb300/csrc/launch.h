@@ -69,10 +69,11 @@ cudaError_t launch_base_p(const float* p, int64_t nq, float gp0, float gp1, floa
                           float* out, cudaStream_t st);
 cudaError_t launch_recall_curve(const int64_t* ids_k, const int64_t* ids_t, int64_t nq, int K,
                                 int T, int32_t* counts, cudaStream_t st);
+// Exhaustive search: ws holds nslices x nq x k 8-byte keys.
 int exact_workspace_slices(int64_t n, int64_t nq, int k, int num_sms);
 cudaError_t launch_exact(const float* base, int64_t n, int d, int d_pad, const float* q,
-                         const float* p, int64_t nq, int k, int nslices, float* part_d,
-                         int32_t* part_i, int64_t* out_ids, float* out_dist, cudaStream_t st);
+                         const float* p, int64_t nq, int k, int nslices, void* ws,
+                         int64_t* out_ids, float* out_dist, cudaStream_t st);
 
 // per-storage-type entry points (defined in wsearch_<type>.cu and csearch_<type>_w<warps>.cu)
 cudaError_t launch_wsearch_f32(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
