@@ -537,7 +537,7 @@ int uhnsw_build_graph(const float* base, int64_t n, int32_t d, int32_t metric, i
 /*
  * The same construction on the current CUDA device (Section 2.2's graphs,
  * built for inputs too large for the host builder).  Nodes are inserted in
- * batches: a batch searches the graph of the nodes before it (one warp per
+ * batches: a batch searches the graph of the nodes before it (one block per
  * new node, efConstruction beam, the neighbour heuristic), then its reverse
  * links are applied row by row, re-selecting a row past its cap with the
  * heuristic.  A batch holds 1/16 of the nodes already inserted (1 to 65,536),

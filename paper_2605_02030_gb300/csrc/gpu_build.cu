@@ -4,15 +4,15 @@
 //
 // The published HNSW insertion, applied to batches of nodes at once:
 //   - nodes are inserted in id order; node 0 is the first entry point;
-//   - a batch [s, e) searches the graph of nodes [0, s): one warp per new
+//   - a batch [s, e) searches the graph of nodes [0, s): a block per new
 //     node runs the greedy descent (beam 1) above the node's level, then at
 //     each level from min(top, level) down to 0 a beam search of width
 //     efConstruction whose entry set is the whole result of the level above,
 //     and keeps at most M links chosen by the neighbour heuristic (a
 //     candidate is kept only if strictly nearer to the new node than to every
 //     link already kept);
-//   - the reverse links go to a per-row incoming buffer; after the batch, one
-//     warp per touched row appends them, or, past the row's cap (2M at layer
+//   - the reverse links go to a per-row incoming buffer; after the batch, a
+//     block per touched row appends them, or, past the row's cap (2M at layer
 //     0, M above), re-selects the row with the heuristic over its old links
 //     and the incoming ones, ordered by (distance, id);
 //   - the entry point moves to the first node of a new top level.
@@ -37,12 +37,12 @@
 
 #include "uhnsw.h"
 #include "uhnsw_internal.h"
-#include "warp_kernels.cuh"
+#include "coop_kernels.cuh"
 
 namespace uhnsw_dev {
 namespace {
 
-constexpr int kBuildWarps = 4;   // warps (new nodes) per block
+constexpr int kBuildWarps = 4;   // warps per block of the reverse-link kernel
 constexpr int kInCap = 128;      // incoming links buffered per row and batch
 
 struct BuildArgs {
@@ -58,77 +58,9 @@ struct BuildArgs {
   int32_t* touched_n;
   int32_t* err;            // [0] error code, [1] dropped incoming links
   int64_t n, rows;
-  int32_t d_pad, metric, M, M0, efc, hb;
+  int32_t d_pad, metric, M, M0, efc;
   float bp;                // the p of metric 5
 };
-
-// Sum of the base-metric terms of two rows by a team of 8 lanes (each lane
-// 4 elements per 32), combined over the team by a butterfly: every lane of
-// the team ends with the sum.  b may point to shared memory.  Metric 5 takes
-// |d_j|^bp through the fast power intrinsic.
-__device__ __forceinline__ float team_dist(const float* __restrict__ a, const float* b, int d_pad,
-                                           int lt, int metric, float bp) {
-  float acc = 0.f;
-  for (int j = lt * 4; j < d_pad; j += 32) {
-    const float4 x = *reinterpret_cast<const float4*>(a + j);
-    const float4 y = *reinterpret_cast<const float4*>(b + j);
-    const float t[4] = {x.x - y.x, x.y - y.y, x.z - y.z, x.w - y.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float v = fabsf(t[e]);
-      acc += metric == UHNSW_BASE_L1    ? v
-             : metric == UHNSW_BASE_L05 ? sqrtf(v)
-             : metric == UHNSW_BASE_L15 ? v * sqrtf(v)
-             : metric == UHNSW_BASE_LP  ? __powf(v, bp)
-                                        : v * v;
-    }
-  }
-  acc += __shfl_xor_sync(kFull, acc, 1);
-  acc += __shfl_xor_sync(kFull, acc, 2);
-  acc += __shfl_xor_sync(kFull, acc, 4);
-  return acc;
-}
-
-// Distances from the row `x` (shared or global) to rows ids[0..m) into out.
-__device__ __forceinline__ void warp_dists(const BuildArgs& a, const float* x, const uint32_t* ids,
-                                           float* out, int m) {
-  const int lane = threadIdx.x & 31, team = lane >> 3, lt = lane & 7;
-  for (int i0 = 0; i0 < m; i0 += 4) {
-    const int i = min(i0 + team, m - 1);
-    const int64_t v = chk_idx((int64_t)(ids[i] & kIdMask), a.n, 20, a.err);
-    const float s = team_dist(a.X + v * a.d_pad, x, a.d_pad, lt, a.metric, a.bp);
-    if (lt == 0 && i0 + team < m) out[i0 + team] = s;
-  }
-  __syncwarp();
-}
-
-// Neighbour heuristic over the ascending candidates (cd, ci)[0..nc): a
-// candidate is kept only if its distance to the base point is below its
-// distance to every candidate already kept; at most m kept, into sel.
-__device__ int warp_select(const BuildArgs& a, const float* cd, const uint32_t* ci, int nc, int m,
-                           int32_t* sel) {
-  const int lane = threadIdx.x & 31, team = lane >> 3, lt = lane & 7;
-  int r = 0;
-  for (int i = 0; i < nc && r < m; ++i) {
-    const int64_t c = chk_idx((int64_t)(ci[i] & kIdMask), a.n, 21, a.err);
-    const float dc = cd[i];
-    const float* xc = a.X + c * a.d_pad;
-    bool keep = true;
-    for (int j0 = 0; j0 < r && keep; j0 += 4) {
-      const int j = min(j0 + team, r - 1);
-      const int64_t s = chk_idx((int64_t)sel[j], a.n, 22, a.err);
-      const float ds = team_dist(xc, a.X + s * a.d_pad, a.d_pad, lt, a.metric, a.bp);
-      const bool bad = j0 + team < r && !(dc < ds);
-      keep = !__any_sync(kFull, bad);
-    }
-    if (keep) {
-      if (lane == 0) sel[r] = (int32_t)c;
-      ++r;
-    }
-    __syncwarp();
-  }
-  return r;
-}
 
 __device__ __forceinline__ const int32_t* adj_row(const BuildArgs& a, int32_t v, int l, int* deg) {
   if (l == 0) {
@@ -144,106 +76,6 @@ __device__ __forceinline__ const int32_t* adj_row(const BuildArgs& a, int32_t v,
   return a.up_adj + chk_idx((int64_t)r + l - 1, a.rows, 25, a.err) * a.M;
 }
 
-// Per-warp shared memory of the insertion kernel.
-struct BuildSmem {
-  int qv, wd0, wi0, wd1, wi1, hash, cd, ci, sd, si, sel, total;
-  __host__ __device__ BuildSmem(int d_pad, int efc, int hb, int cm, int m0) {
-    int o = 0;
-    qv = o; o += align16(d_pad * 4);
-    wd0 = o; o += align16(efc * 4);
-    wi0 = o; o += align16(efc * 4);
-    wd1 = o; o += align16(efc * 4);
-    wi1 = o; o += align16(efc * 4);
-    hash = o; o += align16((1 << hb) * 4);
-    cd = o; o += align16(cm * 4);
-    ci = o; o += align16(cm * 4);
-    sd = o; o += align16(cm * 4);
-    si = o; o += align16(cm * 4);
-    sel = o; o += align16(m0 * 4);
-    total = o;
-  }
-};
-
-// SEARCH-LAYER at level l with beam ef from the entry set held in (*wd, *wi)
-// [0..*nw) (ascending, flags clear); on return the result set is there,
-// ascending, flags clear.  The two list buffers swap roles as the merge runs.
-__device__ void warp_search_layer(const BuildArgs& a, const float* qv, int l, int ef,
-                                  float** wd, uint32_t** wi, float** xd, uint32_t** xi, int* nw,
-                                  int32_t* tab, float* cd, uint32_t* ci, float* sd, uint32_t* si) {
-  const int lane = threadIdx.x & 31;
-  const int H = 1 << a.hb;
-  for (int j = lane; j < H; j += 32) tab[j] = kEmpty;
-  __syncwarp();
-  for (int j = lane; j < *nw; j += 32) hash_insert(tab, a.hb, (int32_t)((*wi)[j] & kIdMask), a.err);
-  __syncwarp();
-  int hcount = *nw, bn = *nw, first = 0;
-  float* bdc = *wd;
-  uint32_t* bic = *wi;
-  float* bdn = *xd;
-  uint32_t* bin = *xi;
-  const int64_t max_steps = a.n + 16;
-  for (int64_t step = 0; first < bn; ++step) {
-    if (step >= max_steps) {
-      if (lane == 0) set_error(a.err, UHNSW_ECAPACITY);
-      break;
-    }
-    // the first unexpanded entry of W, marked expanded
-    int par = -1;
-    for (int b0 = first; b0 < bn && par < 0; b0 += 32) {
-      const int pos = b0 + lane;
-      const unsigned ball = __ballot_sync(kFull, pos < bn && !(bic[pos] & kExpanded));
-      if (ball) {
-        const int src = b0 + __ffs(ball) - 1;
-        par = (int)(bic[src] & kIdMask);
-        __syncwarp();
-        if (lane == 0) bic[src] |= kExpanded;
-      }
-    }
-    __syncwarp();
-    if (par < 0) break;
-    int deg = 0;
-    const int32_t* row = adj_row(a, par, l, &deg);
-    int m = 0;
-    for (int b0 = 0; b0 < deg; b0 += 32) {
-      const int j = b0 + lane;
-      const int32_t v = j < deg ? row[j] : -1;
-      const bool fresh = v >= 0 && v < a.n && hash_insert(tab, a.hb, v, a.err);
-      warp_append(fresh, (uint32_t)v, ci, m, deg, a.err);
-    }
-    __syncwarp();
-    if (m > 0) warp_dists(a, qv, ci, cd, m);
-    const int mk = bn == ef ? warp_reject(cd, ci, m, bdc[bn - 1], (int32_t)(bic[bn - 1] & kIdMask))
-                            : m;
-    int nfirst = 0;
-    const int nbn = warp_merge(bdc, bic, bn, cd, ci, mk, sd, si, bdn, bin, ef, &nfirst);
-    {
-      float* t0 = bdc;
-      bdc = bdn;
-      bdn = t0;
-      uint32_t* t1 = bic;
-      bic = bin;
-      bin = t1;
-    }
-    hcount += m;
-    if (hcount > (H >> 1)) {
-      for (int j = lane; j < H; j += 32) tab[j] = kEmpty;
-      __syncwarp();
-      for (int j = lane; j < nbn; j += 32) hash_insert(tab, a.hb, (int32_t)(bic[j] & kIdMask), a.err);
-      __syncwarp();
-      hcount = nbn;
-    }
-    bn = nbn;
-    first = nfirst;
-  }
-  for (int j = lane; j < bn; j += 32) bic[j] &= kIdMask;
-  __syncwarp();
-  *wd = bdc;
-  *wi = bic;
-  *xd = bdn;
-  *xi = bin;
-  *nw = bn;
-}
-
 // Queues the reverse link (row r <- u) for the batch's second phase.
 __device__ __forceinline__ void push_incoming(const BuildArgs& a, int64_t r, int32_t u) {
   const int pos = atomicAdd(&a.inc_cnt[r], 1);
@@ -255,80 +87,343 @@ __device__ __forceinline__ void push_incoming(const BuildArgs& a, int64_t r, int
   else atomicAdd(&a.err[1], 1);  // dropped: the row had more incoming links than the buffer
 }
 
-// Phase 1 of a batch: one warp per new node u in [s, e).
-__global__ void __launch_bounds__(kBuildWarps * 32) build_insert_kernel(BuildArgs a, int64_t s, int64_t e,
-                                                                       int32_t ep, int32_t top) {
+// Phase 1 of a batch: one block of NW + 1 warps per new node, with the step of
+// the cooperative search (coop_kernels.cuh): NW warps sum the rows of a step,
+// the last merges W, and every warp picks the next parent.  An insertion is a
+// chain of about efConstruction such steps, and the schedule runs about 150
+// batches one after the other for 50,000 nodes, so the chain is what bounds
+// the build.  Eight, four or two distance warps are taken by the size of the
+// batch, the most with which all its nodes are resident at once; two past that
+// (one warp per node, without the step's overlap, took 1.5 times as long at
+// 1M x 128 and 2.1 times at 60k x 960).  Rows are summed by teams of 8 lanes,
+// 4 elements a lane and group of 32, two rows at a time.
+
+// acc + the base-metric terms of four elements, added in order.
+template <int METRIC>
+__device__ __forceinline__ float build_terms(float acc, const float4& x, const float4& y, float bp) {
+  const float t[4] = {x.x - y.x, x.y - y.y, x.z - y.z, x.w - y.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float v = fabsf(t[e]);
+    if (METRIC == UHNSW_BASE_L1) acc = __fadd_rn(acc, v);
+    else if (METRIC == UHNSW_BASE_L05) acc = __fadd_rn(acc, sqrtf(v));
+    else if (METRIC == UHNSW_BASE_L15) acc = fmaf(v, sqrtf(v), acc);
+    else if (METRIC == UHNSW_BASE_LP) acc = __fadd_rn(acc, __powf(v, bp));
+    else acc = fmaf(v, v, acc);
+  }
+  return acc;
+}
+
+// Sums of rows ra and rb against y (shared or global) by a team of 8 lanes,
+// four 32-element groups of both rows loaded before they are summed.
+template <int METRIC>
+__device__ __forceinline__ void build_dist2(const float* __restrict__ ra,
+                                            const float* __restrict__ rb, const float* y, int d_pad,
+                                            int lt, float bp, float& sa, float& sb) {
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  sa = sb = 0.f;
+  for (int j0 = lt * 4; j0 < d_pad; j0 += 128) {
+    float4 xa[4], xb[4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const int j = j0 + 32 * g;
+      xa[g] = j < d_pad ? __ldg(reinterpret_cast<const float4*>(ra + j)) : z;
+      xb[g] = j < d_pad ? __ldg(reinterpret_cast<const float4*>(rb + j)) : z;
+    }
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const int j = j0 + 32 * g;
+      if (j < d_pad) {
+        const float4 yy = *reinterpret_cast<const float4*>(y + j);
+        sa = build_terms<METRIC>(sa, xa[g], yy, bp);
+        sb = build_terms<METRIC>(sb, xb[g], yy, bp);
+      }
+    }
+  }
+#pragma unroll
+  for (int off = 1; off < 8; off <<= 1) {
+    sa += __shfl_xor_sync(kFull, sa, off);
+    sb += __shfl_xor_sync(kFull, sb, off);
+  }
+}
+__device__ __forceinline__ void build_dist2_metric(int metric, const float* ra, const float* rb,
+                                                   const float* y, int d_pad, int lt, float bp,
+                                                   float& sa, float& sb) {
+  switch (metric) {
+    case UHNSW_BASE_L1: build_dist2<1>(ra, rb, y, d_pad, lt, bp, sa, sb); break;
+    case UHNSW_BASE_L2: build_dist2<2>(ra, rb, y, d_pad, lt, bp, sa, sb); break;
+    case UHNSW_BASE_L05: build_dist2<3>(ra, rb, y, d_pad, lt, bp, sa, sb); break;
+    case UHNSW_BASE_L15: build_dist2<4>(ra, rb, y, d_pad, lt, bp, sa, sb); break;
+    default: build_dist2<5>(ra, rb, y, d_pad, lt, bp, sa, sb); break;
+  }
+}
+
+// Neighbour heuristic by a block of G warps over the ascending candidates
+// W[0 .. nw): a candidate is kept only if its distance to the base point is
+// below its distance to every candidate already kept; at most m kept.  G
+// candidates at a time: each warp checks one against those kept so far, and
+// the survivors are taken in order, each first checked against those just
+// taken.  Lane j of every warp ends with kept[i] = the (32 i + j)-th; returns
+// their number.  state: [2][G] shared ints.
+template <int G, int KC>
+__device__ __forceinline__ int block_select(const BuildArgs& a, const unsigned long long* W, int nw,
+                                            int m, uint32_t (&kept)[KC], int32_t* state) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, team = lane >> 3, lt = lane & 7;
+  auto kept_row = [&](int j) {
+    uint32_t v = __shfl_sync(kFull, kept[0], j & 31);
+#pragma unroll
+    for (int c = 1; c < KC; ++c) {
+      const uint32_t w = __shfl_sync(kFull, kept[c], j & 31);
+      if (j >> 5 == c) v = w;
+    }
+    return a.X + (int64_t)v * a.d_pad;
+  };
+  int r = 0, ph = 0;
+  for (int i0 = 0; i0 < nw && r < m; i0 += G) {
+    const int i = i0 + warp;
+    const unsigned long long x = i < nw ? W[i] : kNoKey;
+    const float dc = key_dist(x);
+    const float* xc = a.X + (int64_t)(i < nw ? key_id(x) : 0) * a.d_pad;
+    bool keep = i < nw;
+    for (int j0 = 0; j0 < r && keep; j0 += 8) {
+      const float* ra = kept_row(min(j0 + team, r - 1));
+      const float* rb = kept_row(min(j0 + 4 + team, r - 1));
+      float sa, sb;
+      build_dist2_metric(a.metric, ra, rb, xc, a.d_pad, lt, a.bp, sa, sb);
+      keep = !__any_sync(kFull, !(dc < sa) || !(dc < sb));
+    }
+    if (lane == 0) state[ph * G + warp] = keep;
+    __syncthreads();
+    unsigned mask = __ballot_sync(kFull, lane < G && state[ph * G + min(lane, G - 1)] != 0);
+    ph ^= 1;
+    while (mask && r < m) {
+      const uint32_t id = key_id(W[i0 + __ffs(mask) - 1]);
+#pragma unroll
+      for (int c = 0; c < KC; ++c)
+        if (r == 32 * c + lane) kept[c] = id;
+      ++r;
+      mask &= mask - 1;
+      if (!mask || r >= m) break;
+      bool still = (mask >> warp) & 1u;
+      if (still) {
+        const float* xs = a.X + (int64_t)id * a.d_pad;
+        float sa, sb;
+        build_dist2_metric(a.metric, xs, xs, xc, a.d_pad, lt, a.bp, sa, sb);
+        still = dc < sa;
+      }
+      if (lane == 0) state[ph * G + warp] = still;
+      __syncthreads();
+      mask = __ballot_sync(kFull, lane < G && state[ph * G + min(lane, G - 1)] != 0);
+      ph ^= 1;
+    }
+  }
+  return r;
+}
+
+struct BuildInsertLayout {
+  int qv, W, tab, ck0, ck1, nk, sk, wl, cnt, pub, total;
+  __host__ __device__ BuildInsertLayout(int d_pad, int efc, int hb, int slots, int warps) {
+    const int keys = (slots + 63) / 64 * 64;
+    int o = 0;
+    qv = o; o += align16(d_pad * 4);
+    W = o; o += align16(efc * 8);
+    tab = o; o += (1 << hb) * 4;
+    ck0 = o; o += keys * 8;
+    ck1 = o; o += keys * 8;
+    nk = o; o += keys * 8;
+    sk = o; o += (keys + 32) * 8;
+    wl = o; o += warps * 32 * 4;
+    cnt = o; o += align16(2 * warps * 4);
+    pub = o; o += 2 * (int)sizeof(CoopPub);
+    total = o;
+  }
+};
+
+template <int NW>
+__global__ void __launch_bounds__((NW + 1) * 32, (NW >= 8 ? 1 : NW >= 4 ? 4 : 7))
+    build_insert_kernel(const BuildArgs a, int64_t s, int32_t ep, int32_t top, int hb) {
+  constexpr int THREADS = (NW + 1) * 32;
   extern __shared__ __align__(16) unsigned char smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int cm = max(a.M0, 32);
-  const BuildSmem L(a.d_pad, a.efc, a.hb, cm, a.M0);
-  unsigned char* ws = smem + (size_t)warp * L.total;
-  float* qv = reinterpret_cast<float*>(ws + L.qv);
-  int32_t* tab = reinterpret_cast<int32_t*>(ws + L.hash);
-  float* cd = reinterpret_cast<float*>(ws + L.cd);
-  uint32_t* ci = reinterpret_cast<uint32_t*>(ws + L.ci);
-  float* sd = reinterpret_cast<float*>(ws + L.sd);
-  uint32_t* si = reinterpret_cast<uint32_t*>(ws + L.si);
-  int32_t* sel = reinterpret_cast<int32_t*>(ws + L.sel);
-  const int64_t nwarps = (int64_t)gridDim.x * kBuildWarps;
-  for (int64_t u = s + (int64_t)blockIdx.x * kBuildWarps + warp; u < e; u += nwarps) {
-    const float* xu = a.X + u * a.d_pad;
-    for (int j = lane; j < a.d_pad; j += 32) qv[j] = xu[j];
+  const int spw = (a.M0 + NW - 1) / NW, total = spw * NW, keys = (total + 63) / 64 * 64;
+  const BuildInsertLayout L(a.d_pad, a.efc, hb, total, NW + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int team = lane >> 3, lt = lane & 7;
+  const bool merger = warp == NW;
+  float* qv = reinterpret_cast<float*>(smem + L.qv);
+  unsigned long long* W = reinterpret_cast<unsigned long long*>(smem + L.W);
+  int32_t* tab = reinterpret_cast<int32_t*>(smem + L.tab);
+  unsigned long long* nk = reinterpret_cast<unsigned long long*>(smem + L.nk);
+  unsigned long long* sk = reinterpret_cast<unsigned long long*>(smem + L.sk);
+  uint32_t* wl = reinterpret_cast<uint32_t*>(smem + L.wl) + warp * 32;
+  int32_t* fresh_of = reinterpret_cast<int32_t*>(smem + L.cnt);
+  CoopPub* pub = reinterpret_cast<CoopPub*>(smem + L.pub);
+  auto ckbuf = [&](int i) {
+    return reinterpret_cast<unsigned long long*>(smem + (i ? L.ck1 : L.ck0));
+  };
+  const int64_t u = s + blockIdx.x;
+  const int H = 1 << hb;
+  for (int j = tid; j < a.d_pad; j += THREADS) qv[j] = a.X[u * a.d_pad + j];
+  for (int j = tid; j < 2 * keys; j += THREADS)
+    ckbuf(j >= keys)[j >= keys ? j - keys : j] = kNoKey;
+  __syncthreads();
+
+  // this warp's slots [b, b + 32) of a step (lane i: link v, -1: none), those
+  // not seen at this level summed into out, the others emptied
+  auto sum_slots = [&](int b, int32_t v, bool filter, unsigned long long* out) {
+    const int cnt = min(32, spw - b);
+    unsigned long long* o = out + warp * spw + b;
+    const bool fresh = v >= 0 && v < a.n && (!filter || hash_insert(tab, hb, v, a.err));
+    const unsigned mask = __ballot_sync(kFull, fresh);
+    const int nf = __popc(mask);
+    if (fresh) wl[__popc(mask & lanemask_lt())] = (uint32_t)v;
+    if (lane >= nf && lane < cnt) o[lane] = kNoKey;
     __syncwarp();
-    float* wd = reinterpret_cast<float*>(ws + L.wd0);
-    uint32_t* wi = reinterpret_cast<uint32_t*>(ws + L.wi0);
-    float* xd = reinterpret_cast<float*>(ws + L.wd1);
-    uint32_t* xi = reinterpret_cast<uint32_t*>(ws + L.wi1);
-    if (lane == 0) ci[0] = (uint32_t)ep;
-    __syncwarp();
-    warp_dists(a, qv, ci, cd, 1);
-    if (lane == 0) {
-      wd[0] = cd[0];
-      wi[0] = (uint32_t)ep;
+    for (int i0 = 0; i0 < nf; i0 += 8) {
+      const int ia = i0 + team, ib = ia + 4;
+      const uint32_t da = wl[min(ia, nf - 1)], db = wl[min(ib, nf - 1)];
+      float sa, sb;
+      build_dist2_metric(a.metric, a.X + (int64_t)da * a.d_pad, a.X + (int64_t)db * a.d_pad, qv,
+                         a.d_pad, lt, a.bp, sa, sb);
+      if (lt == 0 && ia < nf) o[ia] = make_key(sa, da);
+      if (lt == 0 && ib < nf) o[ib] = make_key(sb, db);
     }
     __syncwarp();
-    int nw = 1;
-    const int lu = a.lv[u];
-    for (int l = top; l > lu; --l)  // greedy descent: beam 1
-      warp_search_layer(a, qv, l, 1, &wd, &wi, &xd, &xi, &nw, tab, cd, ci, sd, si);
-    for (int l = min(top, lu); l >= 0; --l) {
-      warp_search_layer(a, qv, l, a.efc, &wd, &wi, &xd, &xi, &nw, tab, cd, ci, sd, si);
-      const int r = warp_select(a, wd, wi, nw, a.M, sel);
-      int deg = 0;
-      int32_t* row = const_cast<int32_t*>(adj_row(a, (int32_t)u, l, &deg));
-      for (int j = lane; j < deg; j += 32) row[j] = j < r ? sel[j] : -1;
-      for (int j = lane; j < r; j += 32) {
-        const int32_t v = sel[j];
+    return nf;
+  };
+  // one step's share of this warp: the links of node v at level l
+  auto expand = [&](int32_t v, int l, bool filter, unsigned long long* out) {
+    int deg = 0;
+    const int32_t* row = adj_row(a, v, l, &deg);
+    int nf = 0;
+    for (int b = 0; b < spw; b += 32) {
+      const int f = warp * spw + b + lane;
+      nf += sum_slots(b, b + lane < spw && f < deg ? row[f] : -1, filter, out);
+    }
+    return nf;
+  };
+
+  // beam 1 down to the node's own level
+  int ph = 0;
+  if (warp == 0) sum_slots(0, lane == 0 ? ep : -1, false, ckbuf(0));
+  __syncthreads();
+  unsigned long long curk = ckbuf(0)[0];
+  const int lu = a.lv[u];
+  const int64_t max_steps = ((int64_t)top + 1) * (a.n + 16);
+  int64_t step = 0;
+  for (int l = top; l > lu && step < max_steps; ++step) {
+    ph ^= 1;
+    if (!merger) expand((int32_t)key_id(curk), l, false, ckbuf(ph));
+    __syncthreads();
+    unsigned long long mn = kNoKey;
+    for (int b = lane; b < total; b += 32) mn = ckbuf(ph)[b] < mn ? ckbuf(ph)[b] : mn;
+    mn = warp_min_key(mn);
+    if (mn < curk) curk = mn;
+    else --l;
+  }
+  if (tid == 0) W[0] = curk;
+  int nw = 1;
+  for (int l = min(top, lu); l >= 0; --l) {
+    // SEARCH-LAYER of width efConstruction from the entry set W
+    __syncthreads();
+    for (int j = tid; j < H / 4; j += THREADS)
+      reinterpret_cast<int4*>(tab)[j] = make_int4(kEmpty, kEmpty, kEmpty, kEmpty);
+    for (int j = tid; j < 2 * keys; j += THREADS)
+      ckbuf(j >= keys)[j >= keys ? j - keys : j] = kNoKey;
+    __syncthreads();
+    for (int j = tid; j < nw; j += THREADS) hash_insert(tab, hb, (int32_t)key_id(W[j]), a.err);
+    if (merger) {
+      if (lane == 0) {
+        pub[0].uk[0] = W[0];
+        pub[0].pos[0] = 0;
+        pub[0].bn = nw;
+        pub[0].last = kNoKey;
+      }
+      __syncwarp();
+      coop_merge_step(W, a.efc, 1, ckbuf(0), 0, &pub[0], &pub[1], 0, 0, nk, sk);
+    }
+    __syncthreads();
+    ph = 1;
+    int hcount = nw, nWp = 0, jn = 0;
+    uint32_t par = 0;
+    int npar = coop_select(ckbuf(ph), total, &pub[ph], 1, a.efc, nWp, jn, par);
+    for (int64_t st = 0; npar > 0; ++st) {
+      if (st >= a.n + 16) {
+        if (tid == 0) set_error(a.err, UHNSW_ECAPACITY);
+        break;
+      }
+      if (merger)
+        coop_merge_step(W, a.efc, 1, ckbuf(ph), total, &pub[ph], &pub[ph ^ 1], nWp, jn, nk, sk);
+      if (hcount > (H >> 1)) {
+        __syncthreads();
+        hcount = pub[ph ^ 1].bn;
+        for (int j = tid; j < H / 4; j += THREADS)
+          reinterpret_cast<int4*>(tab)[j] = make_int4(kEmpty, kEmpty, kEmpty, kEmpty);
+        __syncthreads();
+        for (int j = tid; j < hcount; j += THREADS)
+          hash_insert(tab, hb, (int32_t)key_id(W[j]), a.err);
+        __syncthreads();
+      }
+      if (!merger) {
+        const int nf = expand((int32_t)__shfl_sync(kFull, par, 0), l, true, ckbuf(ph ^ 1));
+        if (lane == 0) fresh_of[(ph ^ 1) * NW + warp] = nf;
+      }
+      __syncthreads();
+      ph ^= 1;
+      hcount += (int)__reduce_add_sync(kFull, lane < NW ? (unsigned)fresh_of[ph * NW + lane] : 0u);
+      npar = coop_select(ckbuf(ph), total, &pub[ph], 1, a.efc, nWp, jn, par);
+    }
+    nw = pub[ph].bn;
+    for (int j = tid; j < nw; j += THREADS) W[j] &= ~1ull;
+    __syncthreads();
+
+    uint32_t kept[2] = {0, 0};
+    const int r = block_select<NW + 1, 2>(a, W, nw, a.M, kept, reinterpret_cast<int32_t*>(nk));
+    int deg = 0;
+    int32_t* row = const_cast<int32_t*>(adj_row(a, (int32_t)u, l, &deg));
+    if (warp == 0) {
+      for (int j = lane; j < deg; j += 32) {
+        const int32_t v = (int32_t)(j < 32 ? kept[0] : kept[1]);  // (M <= 64 links)
+        row[j] = j < r ? v : -1;
+        if (j >= r) continue;
         const int32_t off = l == 0 ? 0 : a.up_off[v];
-        if (off < 0) {            // a level-l link to a node below level l
+        if (off < 0) {  // a level-l link to a node below level l
           set_error(a.err, UHNSW_EINVAL);
           continue;
         }
         const int64_t rid = l == 0 ? (int64_t)v : a.n + (int64_t)off + l - 1;
         push_incoming(a, chk_idx(rid, a.n + a.rows, 29, a.err), (int32_t)u);
       }
-      __syncwarp();
     }
   }
 }
 
-// Phase 2 of a batch: one warp per row that received links.
-__global__ void __launch_bounds__(kBuildWarps * 32) build_reverse_kernel(BuildArgs a) {
+// Phase 2 of a batch: one block per row that received links; a row past its
+// cap is re-selected by all its warps, others only take the new links.
+struct BuildReverseLayout {
+  int qv, ui, key, sorted, state, total;
+  __host__ __device__ BuildReverseLayout(int d_pad, int M0) {
+    const int ucap = M0 + kInCap;
+    int o = 0;
+    qv = o; o += align16(d_pad * 4);
+    ui = o; o += align16(ucap * 4);
+    key = o; o += align16(ucap * 8);
+    sorted = o; o += align16(ucap * 8);
+    state = o; o += 2 * kBuildWarps * 4;
+    total = o;
+  }
+};
+
+__global__ void __launch_bounds__(kBuildWarps * 32) build_reverse_kernel(const BuildArgs a) {
+  constexpr int THREADS = kBuildWarps * 32;
   extern __shared__ __align__(16) unsigned char smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ucap = a.M0 + kInCap;
-  // per warp: owner row, union ids / distances, sorted copy, selection
-  const int per = align16(a.d_pad * 4) + 4 * align16(ucap * 4) + align16(a.M0 * 4);
-  unsigned char* ws = smem + (size_t)warp * per;
-  float* qv = reinterpret_cast<float*>(ws);
-  uint32_t* ui = reinterpret_cast<uint32_t*>(ws + align16(a.d_pad * 4));
-  float* ud = reinterpret_cast<float*>(ws + align16(a.d_pad * 4) + align16(ucap * 4));
-  uint32_t* oi = reinterpret_cast<uint32_t*>(ws + align16(a.d_pad * 4) + 2 * align16(ucap * 4));
-  float* od = reinterpret_cast<float*>(ws + align16(a.d_pad * 4) + 3 * align16(ucap * 4));
-  int32_t* sel = reinterpret_cast<int32_t*>(ws + align16(a.d_pad * 4) + 4 * align16(ucap * 4));
+  const BuildReverseLayout L(a.d_pad, a.M0);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, team = lane >> 3, lt = lane & 7;
+  float* qv = reinterpret_cast<float*>(smem + L.qv);
+  uint32_t* ui = reinterpret_cast<uint32_t*>(smem + L.ui);
+  unsigned long long* key = reinterpret_cast<unsigned long long*>(smem + L.key);
+  unsigned long long* sorted = reinterpret_cast<unsigned long long*>(smem + L.sorted);
   const int total = *a.touched_n;
-  const int nwarps = gridDim.x * kBuildWarps;
-  for (int t = blockIdx.x * kBuildWarps + warp; t < total; t += nwarps) {
+  for (int t = blockIdx.x; t < total; t += gridDim.x) {
     const int64_t r = a.touched[chk_idx(t, a.n + a.rows, 27, a.err)];
     const bool l0 = r < a.n;
     const int64_t v = l0 ? r : a.up_owner[chk_idx(r - a.n, a.rows, 28, a.err)];
@@ -341,46 +436,59 @@ __global__ void __launch_bounds__(kBuildWarps * 32) build_reverse_kernel(BuildAr
       const int j = b0 + lane;
       ne += __popc(__ballot_sync(kFull, j < cap && row[j] >= 0));
     }
-    for (int j = lane; j < ne; j += 32) ui[j] = (uint32_t)row[j];
+    const int nu = ne + nin;
     // incoming links sorted by id, so that the row does not depend on the
     // order in which the warps of phase 1 pushed them
-    for (int j = lane; j < nin; j += 32) {
-      const int32_t x = a.inc[r * kInCap + j];
-      int rank = 0;
-      for (int k = 0; k < nin; ++k) rank += a.inc[r * kInCap + k] < x;
-      ui[ne + rank] = (uint32_t)x;
-    }
-    __syncwarp();
-    const int nu = ne + nin;
-    if (nu <= cap) {
-      for (int j = ne + lane; j < nu; j += 32) row[j] = (int32_t)ui[j];
-    } else {
-      const float* xv = a.X + v * a.d_pad;
-      for (int j = lane; j < a.d_pad; j += 32) qv[j] = xv[j];
-      __syncwarp();
-      warp_dists(a, qv, ui, ud, nu);
-      // order by (distance, id)
-      for (int j = lane; j < nu; j += 32) {
-        const float x = ud[j];
-        const int32_t xi = (int32_t)ui[j];
+    for (int j = tid; j < nin; j += THREADS) key[j] = (uint32_t)a.inc[r * kInCap + j];
+    __syncthreads();
+    for (int j = tid; j < nu; j += THREADS) {
+      if (j < ne) {
+        ui[j] = (uint32_t)row[j];
+      } else {
+        const unsigned long long x = key[j - ne];
         int rank = 0;
-        for (int k = 0; k < nu; ++k) rank += pair_lt(ud[k], (int32_t)ui[k], x, xi);
-        od[rank] = x;
-        oi[rank] = (uint32_t)xi;
+        for (int i = 0; i < nin; ++i) rank += key[i] < x;
+        ui[ne + rank] = (uint32_t)x;
       }
-      __syncwarp();
-      const int rs = warp_select(a, od, oi, nu, cap, sel);
-      for (int j = lane; j < cap; j += 32) row[j] = j < rs ? sel[j] : -1;
     }
-    __syncwarp();
-    if (lane == 0) a.inc_cnt[r] = 0;
-    __syncwarp();
+    __syncthreads();
+    if (nu <= cap) {
+      for (int j = ne + tid; j < nu; j += THREADS) row[j] = (int32_t)ui[j];
+    } else {
+      for (int j = tid; j < a.d_pad; j += THREADS) qv[j] = a.X[v * a.d_pad + j];
+      __syncthreads();
+      for (int i0 = warp * 8; i0 < nu; i0 += kBuildWarps * 8) {
+        const int ia = i0 + team, ib = ia + 4;
+        const uint32_t da = ui[min(ia, nu - 1)], db = ui[min(ib, nu - 1)];
+        float sa, sb;
+        build_dist2_metric(a.metric, a.X + chk_idx(da, a.n, 20, a.err) * a.d_pad,
+                           a.X + chk_idx(db, a.n, 20, a.err) * a.d_pad, qv, a.d_pad, lt, a.bp, sa,
+                           sb);
+        if (lt == 0 && ia < nu) key[ia] = make_key(sa, da);
+        if (lt == 0 && ib < nu) key[ib] = make_key(sb, db);
+      }
+      __syncthreads();
+      // order by (distance, id)
+      for (int j = tid; j < nu; j += THREADS) {
+        const unsigned long long x = key[j];
+        int rank = 0;
+        for (int i = 0; i < nu; ++i) rank += key[i] < x;
+        sorted[rank] = x;
+      }
+      __syncthreads();
+      uint32_t kept[4] = {0, 0, 0, 0};  // (caps of up to 128 links)
+      const int rs = block_select<kBuildWarps, 4>(a, sorted, nu, cap, kept,
+                                                  reinterpret_cast<int32_t*>(smem + L.state));
+      if (warp == 0)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int j = 32 * c + lane;
+          if (j < cap) row[j] = j < rs ? (int32_t)kept[c] : -1;
+        }
+    }
+    if (tid == 0) a.inc_cnt[r] = 0;
+    __syncthreads();
   }
-}
-
-int reverse_smem(int d_pad, int M0) {
-  const int ucap = M0 + kInCap;
-  return kBuildWarps * (align16(d_pad * 4) + 4 * align16(ucap * 4) + align16(M0 * 4));
 }
 
 }  // namespace
@@ -428,12 +536,7 @@ int uhnsw_internal::build_graph_gpu(const float* base, int64_t n, int32_t d, int
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return fail(UHNSW_ECUDA, "uhnsw_build_graph_gpu: %s", cudaGetErrorString(e));
-  const BuildSmem L(d_pad, efc, hb, std::max(M0, 32), M0);
-  const size_t smem1 = (size_t)L.total * kBuildWarps;
-  const size_t smem2 = (size_t)reverse_smem(d_pad, M0);
-  if (smem1 > 227 * 1024 || smem2 > 227 * 1024)
-    return fail(UHNSW_ECAPACITY, "uhnsw_build_graph_gpu: %zu / %zu bytes of shared memory per block",
-                smem1, smem2);
+  const size_t smem2 = (size_t)BuildReverseLayout(d_pad, M0).total;
 
   // device buffers
   float* X = nullptr;
@@ -471,19 +574,34 @@ int uhnsw_internal::build_graph_gpu(const float* base, int64_t n, int32_t d, int
   if (e == cudaSuccess) e = cudaMemset(inc_cnt, 0, nr * 4);
   if (e == cudaSuccess) e = cudaMemset(scal, 0, 64);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(build_insert_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem1);
-  if (e == cudaSuccess)
     e = cudaFuncSetAttribute(build_reverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem2);
-  int occ1 = 0, occ2 = 0;
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ1, build_insert_kernel,
-                                                      kBuildWarps * 32, smem1);
+  int occ2 = 0;
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, build_reverse_kernel,
                                                       kBuildWarps * 32, smem2);
-  if (e != cudaSuccess || occ1 < 1 || occ2 < 1) {
+  // the insertion's forms, most warps first, and the batch sizes up to which
+  // all blocks are resident
+  struct Form {
+    void (*kern)(BuildArgs, int64_t, int32_t, int32_t, int);
+    int warps, hb;
+    size_t smem;
+    int64_t cap;
+  } forms[3] = {{build_insert_kernel<8>, 8, 13, 0, 0},
+                {build_insert_kernel<4>, 4, 12, 0, 0},
+                {build_insert_kernel<2>, 2, 11, 0, 0}};
+  for (Form& f : forms) {
+    f.hb = std::max(f.hb, hb);
+    const int slots = (M0 + f.warps - 1) / f.warps * f.warps;
+    f.smem = BuildInsertLayout(d_pad, efc, f.hb, slots, f.warps + 1).total;
+    int occ = 0;
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem);
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f.kern, (f.warps + 1) * 32, f.smem);
+    f.cap = (int64_t)occ * sms;
+  }
+  if (e != cudaSuccess || occ2 < 1 || forms[2].cap < 1) {
     release();
     return fail(UHNSW_ECUDA, "uhnsw_build_graph_gpu: setup: %s",
                 e != cudaSuccess ? cudaGetErrorString(e) : "kernel does not fit");
@@ -509,7 +627,6 @@ int uhnsw_internal::build_graph_gpu(const float* base, int64_t n, int32_t d, int
   a.M = M;
   a.M0 = M0;
   a.efc = efc;
-  a.hb = hb;
 
   int32_t ep = 0, cur_top = levels[0];
   int64_t s = 1;
@@ -517,13 +634,11 @@ int uhnsw_internal::build_graph_gpu(const float* base, int64_t n, int32_t d, int
     const int64_t b = std::max<int64_t>(1, std::min<int64_t>(65536, s / 16));
     const int64_t end = std::min(n, s + b);
     const int64_t warps = end - s;
-    const int64_t grid1 = std::min<int64_t>((warps + kBuildWarps - 1) / kBuildWarps,
-                                            (int64_t)occ1 * sms);
-    build_insert_kernel<<<(unsigned)grid1, kBuildWarps * 32, smem1>>>(a, s, end, ep, cur_top);
+    const Form& form = warps <= forms[0].cap ? forms[0] : warps <= forms[1].cap ? forms[1] : forms[2];
+    form.kern<<<(unsigned)warps, (form.warps + 1) * 32, form.smem>>>(a, s, ep, cur_top, form.hb);
     e = cudaGetLastError();
     if (e != cudaSuccess) break;
-    const int64_t grid2 = std::min<int64_t>((warps * M * 2 + kBuildWarps - 1) / kBuildWarps,
-                                            (int64_t)occ2 * sms);
+    const int64_t grid2 = std::min<int64_t>(warps * M * 2, (int64_t)occ2 * sms);
     build_reverse_kernel<<<(unsigned)std::max<int64_t>(grid2, 1), kBuildWarps * 32, smem2>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) break;
