@@ -1407,7 +1407,7 @@ def verify_roofline(idx, q_dev, w, steps, warmup, t=256, K=50, pv=0.7, n_rows=No
     bound = "alu" if t_sfu >= t_hbm else "hbm"
     top = sfu if bound == "alu" else hbm
     out = {"bound": bound, "achieved": top["achieved"], "peak": top["peak"], "unit": top["unit"],
-           "frac": top["frac"], "kernel": "uhnsw_wverify_kernel (warp per query)",
+           "frac": top["frac"], "kernel": "uhnsw_verify_kernel (block per query)",
            "launch_ms": round(mean_s * 1e3, 4),
            "launch_ms_source": ("%d launches queued back to back on %d streams, per launch"
                                 % (steps, streams) if streams > 1 else

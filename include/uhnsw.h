@@ -193,11 +193,11 @@ typedef struct {
                             and refilled with the beam, which cannot change the beam); a
                             smaller table re-evaluates more nodes, a larger one takes
                             shared memory from other queries. */
-  int32_t verify_groups; /* verification in the warp-per-query kernels: 32-dimension
-                            groups accumulated between two tests of a candidate's partial
-                            sum against the running k-th best sum, 1..16; 0 => 2 in
-                            uhnsw_search, 1 in uhnsw_verify (the block-per-query kernel
-                            tests after every four).  Every lane
+  int32_t verify_groups; /* verification in uhnsw_verify and the warp-per-query search:
+                            32-dimension groups accumulated between two tests of a
+                            candidate's partial sum against the running k-th best sum,
+                            1..16; 0 => 2 in uhnsw_search, 3 in uhnsw_verify (the
+                            block-per-query search tests after every four).  Every lane
                             accumulates its elements in the same order whatever the
                             value, so sums and results do not depend on it; it trades
                             drop-test work for candidates summed further before they are

@@ -937,7 +937,9 @@ extern "C" int uhnsw_verify(uhnsw_index* idx, const float* q, const float* p, co
   a.kappa = opts.kappa;
   a.tau = opts.tau != 0.f ? opts.tau : 0.92f;
   a.mode = opts.verify_mode;
-  a.vgroups = opts.verify_groups > 0 ? opts.verify_groups : 1;
+  // two tests in 128 dimensions: 5,003 queries x 300 candidates take 199 us, 208 with
+  // a test after every group
+  a.vgroups = opts.verify_groups > 0 ? opts.verify_groups : 3;
   a.cmax = kBlock / 8;
   a.vcap = std::max(t, 1);
   a.out_ids = out_ids;
@@ -946,7 +948,7 @@ extern "C" int uhnsw_verify(uhnsw_index* idx, const float* q, const float* p, co
   a.err = idx->err;
   a.cand = cand;
   a.cand_t = t;
-  cudaError_t e = launch_wverify(a, (cudaStream_t)stream);
+  cudaError_t e = launch_verify(a, idx->num_sms, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "uhnsw_verify: launch");
   return UHNSW_OK;
 }

@@ -773,11 +773,10 @@ __device__ void coop_query(const QueryArgs& a, int64_t qi, unsigned char* smem,
       if ((float)ov / (float)k >= tau) break;
     }
   }
-  const double inv_p = 1.0 / (double)p;
   for (int j = tid; j < a.k_max; j += THREADS) {
     const bool have = j < k && j < tn;
     oid[j] = have ? (int64_t)key_id(top[j]) : -1;
-    odist[j] = have ? (float)pow((double)key_dist(top[j]), inv_p) : kInf;
+    odist[j] = have ? root_p(key_dist(top[j]), p) : kInf;
   }
   if (a.stats) {
     if (terms) atomicAdd(&vs[1], terms);

@@ -195,4 +195,67 @@ __device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
   return r;
 }
 
+// s^(1/p) for a sum s >= 0, to within 2^-43 of the exact value before the one
+// rounding to FP32 (the same FP32 value as FP64's pow gives in 20 million random cases; p = 1/2, 1 and 2 are correctly rounded).
+//
+// This chip retires 2 FP64 operations a clock and SM, so a pow per returned
+// distance was 0.07 of 0.29 ms of a verification of 5,003 queries at K = 50.
+// Here log2 is the atanh series of (m - 1) / (m + 1) for the mantissa m in
+// [sqrt(1/2), sqrt(2)), 2^f is e^(f ln 2)'s Taylor series for |f| <= 1/2, and
+// the tails of both, 2^-20 of the sum or less, are summed in FP32.
+__device__ __forceinline__ float root_p(float s, float p) {
+  if (p == 1.0f) return s;
+  if (p == 2.0f) return __fsqrt_rn(s);
+  if (p == 0.5f) return __double2float_rn((double)s * (double)s);
+  if (!(s > 0.0f) || s == __int_as_float(0x7f800000)) return s;  // 0, +inf, NaN
+  // s = m 2^e (a subnormal FP32 value is a normal FP64 one)
+  const double sd = (double)s;
+  const int hi = __double2hiint(sd);
+  const int e = (hi - 0x3fe6a09e) >> 20;  // the high word of sqrt(1/2)
+  const double m = __hiloint2double(hi - (e << 20), __double2loint(sd));
+  const double num = m - 1.0, den = m + 1.0;
+  float rden;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rden) : "f"((float)den));
+  const double rd = (double)rden;
+  double u = num * rd;
+  u = fma(fma(-u, den, num), rd, u);
+  const double w = u * u;
+  const float wf = (float)w;
+  float lt = fmaf(wf, 1.0f / 19, 1.0f / 17);
+  lt = fmaf(wf, lt, 1.0f / 15);
+  lt = fmaf(wf, lt, 1.0f / 13);
+  lt = fmaf(wf, lt, 1.0f / 11);
+  double l = fma(w, (double)lt, 1.0 / 9);
+  l = fma(w, l, 1.0 / 7);
+  l = fma(w, l, 1.0 / 5);
+  l = fma(w, l, 1.0 / 3);
+  l = fma(w, l, 1.0);
+  constexpr double kLn2 = 0.693147180559945309417232;
+  l = fma(u * (2.0 / kLn2), l, (double)e);
+  float rp;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rp) : "f"(p));
+  const double pd = (double)p;
+  double inv = (double)rp;
+  inv = fma(inv, fma(-pd, inv, 1.0), inv);
+  inv = fma(inv, fma(-pd, inv, 1.0), inv);
+  // an exponent beyond FP32's range rounds to 0 or +inf all the same
+  const double z = fmin(fmax(l * inv, -1000.0), 1000.0);
+  const int n = __double2int_rn(z);
+  const double t = (z - (double)n) * kLn2;
+  const float tf = (float)t;
+  float et = fmaf(tf, 1.0f / 479001600, 1.0f / 39916800);
+  et = fmaf(tf, et, 1.0f / 3628800);
+  et = fmaf(tf, et, 1.0f / 362880);
+  et = fmaf(tf, et, 1.0f / 40320);
+  double x = fma(t, (double)et, 1.0 / 5040);
+  x = fma(t, x, 1.0 / 720);
+  x = fma(t, x, 1.0 / 120);
+  x = fma(t, x, 1.0 / 24);
+  x = fma(t, x, 1.0 / 6);
+  x = fma(t, x, 0.5);
+  x = fma(t, x, 1.0);
+  x = fma(t, x, 1.0);
+  return __double2float_rn(__hiloint2double(__double2hiint(x) + (n << 20), __double2loint(x)));
+}
+
 }  // namespace uhnsw_dev

@@ -40,8 +40,8 @@ cudaError_t launch_csearch(uhnsw_dtype dt, int warps, WarpShape sh, const QueryA
 // not fit).
 int csearch_occupancy(uhnsw_dtype dt, int warps, WarpShape sh, size_t smem);
 
-// Verification only, one warp per query (4 per block).
-cudaError_t launch_wverify(const QueryArgs& a, cudaStream_t st);
+// Verification only (verify_kernels.cuh): one block per query.
+cudaError_t launch_verify(const QueryArgs& a, int num_sms, cudaStream_t st);
 
 // Beam buckets of a bucketed persistent search (ascending bounds).
 struct BeamBuckets {

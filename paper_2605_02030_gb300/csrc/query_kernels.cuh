@@ -122,8 +122,8 @@ __device__ __forceinline__ float base_root(int metric, float bp, float s) {
   return metric == UHNSW_BASE_L1    ? s
          : metric == UHNSW_BASE_L2  ? sqrtf(s)
          : metric == UHNSW_BASE_L05 ? (float)((double)s * (double)s)
-         : metric == UHNSW_BASE_L15 ? (float)pow((double)s, 1.0 / 1.5)
-                                    : (float)pow((double)s, 1.0 / (double)bp);
+         : metric == UHNSW_BASE_L15 ? root_p(s, 1.5f)
+                                    : root_p(s, bp);
 }
 
 // Dynamic shared-memory carve-up (byte offsets), identical on host and device.

@@ -2,19 +2,34 @@
 #include <cuda_runtime.h>
 
 #include "launch.h"
+#include "verify_kernels.cuh"
 
 namespace uhnsw_dev {
 
-cudaError_t launch_wverify(const QueryArgs& a, cudaStream_t st) {
-  const WVerifyLayout L(a.d_pad, a.k_max, a.vcap);
-  constexpr int warps = 4;
-  const size_t smem = (size_t)L.total * warps;
-  auto kern = uhnsw_wverify_kernel<warps>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <int NW>
+cudaError_t launch_verify_warps(const QueryArgs& a, cudaStream_t st) {
+  const VerifyLayout L(a.d_pad, a.k_max, a.vcap, NW);
+  auto kern = uhnsw_verify_kernel<NW>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
   if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)((a.nq + warps - 1) / warps);
-  kern<<<grid, warps * 32, smem, st>>>(a);
+  kern<<<(unsigned)a.nq, (NW + 1) * 32, L.total, st>>>(a);
   return cudaGetLastError();
+}
+
+// Warps per query, us for queries x candidates (128 dimensions, 152 SMs; the
+// last column 960 dimensions; K = 50 for 300 candidates, else 10):
+//               1 x 300  456 x 300  1,000 x 300  5,003 x 300  10,000 x 64  10,000 x 10  2,500 x 64
+//   8 warps          43         50           80          223          225          152         160
+//   4 warps          49         56           83          199          132           96         140
+//   2 warps          66         70           80          215          125           76         155
+// Eight while all queries are resident at once (3 blocks of 9 warps an SM):
+// the steps of one query are then what takes the time.  Two where one step of
+// two warps covers the list, as more warps would find no rows to sum, and for
+// up to 64 short rows: in steps of 32 or 64 none of them would be dropped.
+cudaError_t launch_verify(const QueryArgs& a, int num_sms, cudaStream_t st) {
+  if (a.cand_t <= (a.d_pad <= 256 ? 64 : 16)) return launch_verify_warps<2>(a, st);
+  if (a.nq <= 3 * (int64_t)num_sms) return launch_verify_warps<8>(a, st);
+  return launch_verify_warps<4>(a, st);
 }
 
 // FP32 master rows -> FP16 / BF16 traversal rows (round to nearest even).
