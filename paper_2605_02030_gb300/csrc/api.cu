@@ -543,7 +543,7 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
   const int chunks = idx->d_pad / (idx->tdtype == UHNSW_F32 ? 4 : 8);
   WarpShape bsh{0, 0, 0}, wsh{0, 0, 0};
   const bool have_block = pick_block_shape(idx->tdtype, chunks, &bsh);
-  const bool few = nq < (int64_t)idx->num_sms * WarpMinBlocks<float>::value * kWarpsPerBlock;
+  const bool few = nq < (int64_t)idx->num_sms * kWarpSlots;
   const bool have_warp = pick_warp_shape(idx->tdtype, chunks, opts.team_lanes, few, &wsh);
   if (want_warp ? !have_warp : !have_block)
     return fail(UHNSW_ECAPACITY, "uhnsw_search: no kernel shape for d=%d", idx->d);
@@ -666,7 +666,7 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
                                   : std::min(16, std::max(4, (((1 << Lo->a.hash_bits) * 4) / vrow) & ~3));
       const SmemLayout Lw(idx->d_pad, bound, Lo->a.hash_bits, cmax, k_max, 0, sv * vrow);
       const size_t smem = (size_t)Lw.total * kWarpsPerBlock;
-      if (smem <= kSmemMax) {
+      if (4 * (size_t)Lw.total <= kSmemMax) {  // (a limit of the interface, as four per block)
         Lo->shape = wsh;
         Lo->smem = smem;
         Lo->a.cmax = cmax;

@@ -11,16 +11,15 @@
 namespace uhnsw_dev {
 
 // Warp-per-query kernel: TEAM lanes per row, CPL 16-byte chunks per lane,
-// U rows per team loaded per round; 4 warps (queries) per block.
+// U rows per team loaded per round; kWarpsPerBlock warps (queries) per block.
 struct WarpShape {
   int team, cpl, u;
 };
-constexpr int kWarpsPerBlock = 4;
+constexpr int kWarpsPerBlock = 2;
 // The warp kernel's team shape for rows of `chunks` 16-byte chunks.
 // team_pref 0: the narrowest compiled team that covers the row; else the
 // first covering shape with exactly that many lanes.  `few`: the batch has
-// fewer queries than the GPU has warp slots (WarpMinBlocks blocks of
-// kWarpsPerBlock warps per SM).
+// fewer queries than the GPU has warp slots (kWarpSlots per SM).
 bool pick_warp_shape(uhnsw_dtype dt, int chunks, int team_pref, bool few, WarpShape* out);
 cudaError_t launch_wsearch(uhnsw_dtype dt, WarpShape sh, const QueryArgs& a, int grid,
                            size_t smem, cudaStream_t st);

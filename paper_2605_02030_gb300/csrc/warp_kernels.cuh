@@ -678,24 +678,19 @@ __device__ void warp_query(const QueryArgs& a, int64_t qi, unsigned char* ws, co
 // WARPS independent queries per block; a.queue_head set = persistent (each
 // warp pulls the next query index), else query = blockIdx.x * WARPS + warp.
 //
-// Blocks per SM asked of the register allocator: 6 (80 registers, 24 queries
-// per SM).  It measured faster than 8 blocks at 64 registers, whose spill
-// traffic reached DRAM (1.83 vs 1.99 ms and 2.31 vs 2.74 ms per 10,000
-// queries on 1M x 128), and than 7 blocks at 72 registers.  The smaller
-// shared-memory carve-out also leaves a larger L1 for the rows.
-#ifdef UHNSW_WARP_MINB
-template <typename T>
-struct WarpMinBlocks {
-  static constexpr int value = UHNSW_WARP_MINB;
-};
-#else
-template <typename T>
-struct WarpMinBlocks {
-  static constexpr int value = 6;
-};
-#endif
-template <typename T, int TEAM, int CPL, int U, int WARPS, int MINB = WarpMinBlocks<T>::value>
-__global__ void __launch_bounds__(WARPS * 32, MINB) uhnsw_wsearch_kernel(const QueryArgs a) {
+// Warps per SM asked of the register allocator: 24 (80 registers).  It measured
+// faster than 32 warps at 64 registers, whose spill traffic reached DRAM (1.83
+// vs 1.99 ms and 2.31 vs 2.74 ms per 10,000 queries on 1M x 128), and than 28
+// at 72 registers.  The smaller shared-memory carve-out also leaves a larger L1
+// for the rows.
+//
+// Two warps per block: a launch that is not persistent starts the next queries
+// when a block's slowest one is done, which costs less the fewer share it
+// (10,000 FP32 queries, 1M x 128: 2.93 ms with four, 2.86 with two).  With one,
+// the 1 KB that every block reserves takes warps from the SM (3.53 ms).
+constexpr int kWarpSlots = 24;
+template <typename T, int TEAM, int CPL, int U, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, kWarpSlots / WARPS) uhnsw_wsearch_kernel(const QueryArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const SmemLayout L(a.d_pad, a.ef_cap, a.hash_bits, a.cmax, a.k_max, 0, a.stage_bytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
