@@ -552,7 +552,7 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
   // launch's visited table (the two share one region), 4 to 16
   const int vrow = idx->d_pad * 4;
   const int sv_asked = opts.stage_bytes > 0 ? std::max(4, (opts.stage_bytes / vrow) & ~3) : 0;
-  constexpr size_t kSmemMax = 227 * 1024;
+  constexpr size_t kSmemMax = 227 * 1024, kSmSmem = 228 * 1024;
 
   QueryArgs& a = P->a;
   std::memset(&a, 0, sizeof(a));
@@ -668,9 +668,12 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
       const size_t smem = (size_t)Lw.total * kWarpsPerBlock;
       if (4 * (size_t)Lw.total <= kSmemMax) {  // (a limit of the interface, as four per block)
         Lo->shape = wsh;
+        // (the 1 KB that a block reserves beside its own counts too)
+        Lo->shape.most = kSmSmem / (smem + 1024) * kWarpsPerBlock >= (size_t)kWarpSlotsMost;
         Lo->smem = smem;
         Lo->a.cmax = cmax;
         Lo->a.stage_bytes = sv * vrow;
+        Lo->a.lay = Lw;
         Lo->a.sv = sv;
         Lo->grid = (int)((nq + kWarpsPerBlock - 1) / kWarpsPerBlock);
         if (P->persistent) {

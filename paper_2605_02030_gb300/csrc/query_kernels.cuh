@@ -49,6 +49,39 @@ struct GraphDev {
   int32_t deg;
 };
 
+__host__ __device__ inline int align16(int x) { return (x + 15) & ~15; }
+
+// Dynamic shared-memory carve-up (byte offsets), identical on host and device.
+struct SmemLayout {
+  int stage, qs, bd0, bi0, bd1, bi1, hash, cd, ci, sd, si, td0, ti0, td1, ti1, cv, total;
+  SmemLayout() = default;
+  __host__ __device__ SmemLayout(int d_pad, int ef_cap, int hash_bits, int cmax, int k_max,
+                                 int vcap, int stage_bytes = 0) {
+    int o = 0;
+    qs = o; o += align16(d_pad * 4);
+    bd0 = o; o += align16(ef_cap * 4);
+    bi0 = o; o += align16(ef_cap * 4);
+    bd1 = o; o += align16(ef_cap * 4);
+    bi1 = o; o += align16(ef_cap * 4);
+    // The visited table lives during the search, the staged verification rows
+    // after it: they share one region.
+    const int hash_bytes = align16((hash_bits > 0 ? (1 << hash_bits) : 0) * 4);
+    hash = o;
+    stage = o;
+    o += hash_bytes > align16(stage_bytes) ? hash_bytes : align16(stage_bytes);
+    cd = o; o += align16(cmax * 4);
+    ci = o; o += align16(cmax * 4);
+    sd = o; o += align16(cmax * 4);
+    si = o; o += align16(cmax * 4);
+    td0 = o; o += align16(k_max * 4);
+    ti0 = o; o += align16(k_max * 4);
+    td1 = o; o += align16(k_max * 4);
+    ti1 = o; o += align16(k_max * 4);
+    cv = o; o += align16(vcap * 4);
+    total = o;
+  }
+};
+
 struct QueryArgs {
   const float* base32;  // FP32 master copy [n][d_pad]
   const void* trav;     // traversal copy [n][d_pad] in the kernel's element type
@@ -86,11 +119,10 @@ struct QueryArgs {
   int32_t stage_bytes;  // warp kernel: per-warp staging buffer for cp.async row copies
   int32_t sb;           // warp kernel: traversal rows staged per batch
   int32_t sv;           // warp kernel: FP32 rows staged per verification batch (multiple of 4)
+  SmemLayout lay;       // warp kernel: one warp's shared memory
   int32_t vgroups;      // warp kernels' verification: 32-dimension groups between two drop
                         // tests (>= 1); the cooperative kernel tests after every four
 };
-
-__host__ __device__ inline int align16(int x) { return (x + 15) & ~15; }
 
 // Routing of a query (Algorithm 1, lines 1-5): the graph slot it searches,
 // whether it is answered directly (p is that graph's own base p), the slot's
@@ -125,36 +157,6 @@ __device__ __forceinline__ float base_root(int metric, float bp, float s) {
          : metric == UHNSW_BASE_L15 ? root_p(s, 1.5f)
                                     : root_p(s, bp);
 }
-
-// Dynamic shared-memory carve-up (byte offsets), identical on host and device.
-struct SmemLayout {
-  int stage, qs, bd0, bi0, bd1, bi1, hash, cd, ci, sd, si, td0, ti0, td1, ti1, cv, total;
-  __host__ __device__ SmemLayout(int d_pad, int ef_cap, int hash_bits, int cmax, int k_max,
-                                 int vcap, int stage_bytes = 0) {
-    int o = 0;
-    qs = o; o += align16(d_pad * 4);
-    bd0 = o; o += align16(ef_cap * 4);
-    bi0 = o; o += align16(ef_cap * 4);
-    bd1 = o; o += align16(ef_cap * 4);
-    bi1 = o; o += align16(ef_cap * 4);
-    // The visited table lives during the search, the staged verification rows
-    // after it: they share one region.
-    const int hash_bytes = align16((hash_bits > 0 ? (1 << hash_bits) : 0) * 4);
-    hash = o;
-    stage = o;
-    o += hash_bytes > align16(stage_bytes) ? hash_bytes : align16(stage_bytes);
-    cd = o; o += align16(cmax * 4);
-    ci = o; o += align16(cmax * 4);
-    sd = o; o += align16(cmax * 4);
-    si = o; o += align16(cmax * 4);
-    td0 = o; o += align16(k_max * 4);
-    ti0 = o; o += align16(k_max * 4);
-    td1 = o; o += align16(k_max * 4);
-    ti1 = o; o += align16(k_max * 4);
-    cv = o; o += align16(vcap * 4);
-    total = o;
-  }
-};
 
 __device__ __forceinline__ uint32_t dynamic_smem_bytes() {
   uint32_t r;

@@ -675,24 +675,35 @@ __device__ void warp_query(const QueryArgs& a, int64_t qi, unsigned char* ws, co
   if (lane == 0) put_stats(a, qi, nb, v.np, v.terms, nexp, nres, 0, rt.slot + 1, nadj);
 }
 
-// WARPS independent queries per block; a.queue_head set = persistent (each
-// warp pulls the next query index), else query = blockIdx.x * WARPS + warp.
+// Warps per SM asked of the register allocator.  A step of a query is a chain of
+// dependent loads, so more resident queries hide more of it, while spills and a
+// smaller L1 cost; FP32 rows of one or two chunks a lane gain from 32 warps at
+// 64 registers where the launch's shared memory holds that many (small beams),
+// the others run 24 at 80.  32 against 24, 1M x 128 unless stated:
+//   FP32, ef 64, 10,000 queries 2.80 vs 2.93 ms, 4,000 queries 1.44 vs 1.78;
+//     L0.5 and L1 graphs 3.31 vs 4.08; 40k x 180 2.02 vs 2.32; where 32 do not
+//     fit, ef 200 would take 7.50 vs 7.31 and 40k x 50 at ef 300 3.63 vs 3.38;
+//   FP16 (ef 52, width 1) 2.03 vs 1.89, BF16 2.41 vs 1.96, 1M x 96 at ef 64
+//     3.37 vs 2.85.
+// 28 warps at 72 registers are slower than either (FP32 3.50 ms).
 //
-// Warps per SM asked of the register allocator: 24 (80 registers).  It measured
-// faster than 32 warps at 64 registers, whose spill traffic reached DRAM (1.83
-// vs 1.99 ms and 2.31 vs 2.74 ms per 10,000 queries on 1M x 128), and than 28
-// at 72 registers.  The smaller shared-memory carve-out also leaves a larger L1
-// for the rows.
+// The 32-warp form and the rows of three chunks a lane (96 FP16 dimensions) take
+// the shared-memory layout from the launch's arguments, in constant memory: the
+// offsets computed in the kernel stay in registers and spill (1M x 96, ef 512,
+// 10,000 queries 56.1 -> 48.3 ms; 4,000 of mixed ef 19.0 -> 13.1 ms).  For the
+// other 24-warp forms it measured from 7 % slower to 2 % faster.
 //
 // Two warps per block: a launch that is not persistent starts the next queries
 // when a block's slowest one is done, which costs less the fewer share it
 // (10,000 FP32 queries, 1M x 128: 2.93 ms with four, 2.86 with two).  With one,
 // the 1 KB that every block reserves takes warps from the SM (3.53 ms).
-constexpr int kWarpSlots = 24;
+constexpr int kWarpSlots = 24, kWarpSlotsMost = 32;
+
+// WARPS independent queries per block; a.queue_head set = persistent (each
+// warp pulls the next query index), else query = blockIdx.x * WARPS + warp.
 template <typename T, int TEAM, int CPL, int U, int WARPS>
-__global__ void __launch_bounds__(WARPS * 32, kWarpSlots / WARPS) uhnsw_wsearch_kernel(const QueryArgs a) {
+__device__ __forceinline__ void wsearch_block(const QueryArgs& a, const SmemLayout& L) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const SmemLayout L(a.d_pad, a.ef_cap, a.hash_bits, a.cmax, a.k_max, 0, a.stage_bytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if ((uint32_t)(L.total * WARPS) > dynamic_smem_bytes()) {
     if (threadIdx.x == 0) set_error(a.err, UHNSW_ECAPACITY);
@@ -713,6 +724,16 @@ __global__ void __launch_bounds__(WARPS * 32, kWarpSlots / WARPS) uhnsw_wsearch_
     warp_query<T, TEAM, CPL, U>(a, qi, ws, L);
     __syncwarp();
     if (!a.queue_head) break;
+  }
+}
+
+template <typename T, int TEAM, int CPL, int U, int WARPS, int SLOTS>
+__global__ void __launch_bounds__(WARPS * 32, SLOTS / WARPS) uhnsw_wsearch_kernel(const QueryArgs a) {
+  if constexpr (SLOTS == kWarpSlotsMost || CPL == 3) {
+    wsearch_block<T, TEAM, CPL, U, WARPS>(a, a.lay);
+  } else {
+    const SmemLayout L(a.d_pad, a.ef_cap, a.hash_bits, a.cmax, a.k_max, 0, a.stage_bytes);
+    wsearch_block<T, TEAM, CPL, U, WARPS>(a, L);
   }
 }
 

@@ -3,8 +3,8 @@
 
 namespace uhnsw_dev {
 
-#define WLAUNCH_CALL(T, TEAM, CPL, U) wlaunch_one<T, TEAM, CPL, U>(a, grid, smem, st)
-#define WOCC_CALL(T, TEAM, CPL, U) wocc_one<T, TEAM, CPL, U>(smem)
+#define WLAUNCH_CALL(T, TEAM, CPL, U) wlaunch_one<T, TEAM, CPL, U>(sh.most, a, grid, smem, st)
+#define WOCC_CALL(T, TEAM, CPL, U) wocc_one<T, TEAM, CPL, U>(sh.most, smem)
 
 cudaError_t launch_wsearch_f16(WarpShape sh, const QueryArgs& a, int grid, size_t smem,
                                cudaStream_t st) {

@@ -5,9 +5,23 @@
 
 namespace uhnsw_dev {
 
+// The rows whose kernel is also compiled for 32 warps per SM.
+template <typename T, int CPL>
+constexpr bool wsearch_has_most() {
+  return std::is_same<T, float>::value && CPL <= 2;
+}
+
 template <typename T, int TEAM, int CPL, int U>
-cudaError_t wlaunch_one(const QueryArgs& a, int grid, size_t smem, cudaStream_t st) {
-  auto kern = uhnsw_wsearch_kernel<T, TEAM, CPL, U, kWarpsPerBlock>;
+auto wsearch_kernel(bool most) {
+  auto kern = uhnsw_wsearch_kernel<T, TEAM, CPL, U, kWarpsPerBlock, kWarpSlots>;
+  if constexpr (wsearch_has_most<T, CPL>())
+    if (most) kern = uhnsw_wsearch_kernel<T, TEAM, CPL, U, kWarpsPerBlock, kWarpSlotsMost>;
+  return kern;
+}
+
+template <typename T, int TEAM, int CPL, int U>
+cudaError_t wlaunch_one(bool most, const QueryArgs& a, int grid, size_t smem, cudaStream_t st) {
+  auto kern = wsearch_kernel<T, TEAM, CPL, U>(most);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<grid, kWarpsPerBlock * 32, smem, st>>>(a);
@@ -15,8 +29,8 @@ cudaError_t wlaunch_one(const QueryArgs& a, int grid, size_t smem, cudaStream_t 
 }
 
 template <typename T, int TEAM, int CPL, int U>
-int wocc_one(size_t smem) {
-  auto kern = uhnsw_wsearch_kernel<T, TEAM, CPL, U, kWarpsPerBlock>;
+int wocc_one(bool most, size_t smem) {
+  auto kern = wsearch_kernel<T, TEAM, CPL, U>(most);
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return 0;
