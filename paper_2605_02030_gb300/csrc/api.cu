@@ -714,6 +714,7 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
       Lb.a.queue_head = qu->head + b;
       Lb.a.qorder = qu->ws + kBucketOrder;
       Lb.a.qbucket = qu->ws + kBucketInfo + 2 * b;
+      Lb.a.chain = (b > 0 ? 1 : 0) | (b < P->bb.n - 1 ? 2 : 0);
       P->launches.push_back(Lb);
     }
   } else {

@@ -804,12 +804,11 @@ __global__ void __launch_bounds__((NW + 1) * 32, (CoopMinBlocks<CPL, NW>::value)
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int next;
   const CoopLayout L(TEAM * CPL * Elems16<T>::n, a.ef_cap, a.hash_bits, a.cmax, a.k_max, NW + 1);
-  if ((uint32_t)L.total > dynamic_smem_bytes()) {
-    if (threadIdx.x == 0) set_error(a.err, UHNSW_ECAPACITY);
-    return;
-  }
+  chain_begin(a);
+  const bool fits = (uint32_t)L.total <= dynamic_smem_bytes();
+  if (!fits && threadIdx.x == 0) set_error(a.err, UHNSW_ECAPACITY);
   int64_t qi = blockIdx.x;
-  for (;;) {
+  while (fits) {
     if (a.queue_head) {
       if (threadIdx.x == 0) {
         const int slot = atomicAdd(a.queue_head, 1);
@@ -823,6 +822,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, (CoopMinBlocks<CPL, NW>::value)
     __syncthreads();
     if (!a.queue_head) break;
   }
+  chain_end(a);
 }
 
 }  // namespace uhnsw_dev

@@ -17,10 +17,7 @@ struct CoopRows {
 template <typename T, int TEAM, int CPL, int NW>
 cudaError_t claunch_one(const QueryArgs& a, int grid, size_t smem, cudaStream_t st) {
   auto kern = uhnsw_csearch_kernel<T, TEAM, CPL, CoopRows<CPL>::value, NW>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  kern<<<grid, (NW + 1) * 32, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_search_kernel(kern, grid, (NW + 1) * 32, smem, a, st);
 }
 
 // Resident blocks per SM that the registers allow (0: the query failed).

@@ -26,6 +26,26 @@ cudaError_t launch_wsearch(uhnsw_dtype dt, WarpShape sh, const QueryArgs& a, int
                            size_t smem, cudaStream_t st);
 int wsearch_occupancy(uhnsw_dtype dt, WarpShape sh, size_t smem);
 
+// Launches a search kernel; one that follows another of its chain (a.chain) may
+// start before that one's end.
+template <typename K>
+cudaError_t launch_search_kernel(K kern, int grid, int threads, size_t smem, const QueryArgs& a,
+                                 cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute early = {};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &early;
+  cfg.numAttrs = (a.chain & 2) ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
 // Cooperative kernel (coop_kernels.cuh): one query per block, kCoopWarps[i]
 // distance warps and one merge warp.
 constexpr int kCoopForms = 3;

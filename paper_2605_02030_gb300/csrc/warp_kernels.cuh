@@ -729,12 +729,14 @@ __device__ __forceinline__ void wsearch_block(const QueryArgs& a, const SmemLayo
 
 template <typename T, int TEAM, int CPL, int U, int WARPS, int SLOTS>
 __global__ void __launch_bounds__(WARPS * 32, SLOTS / WARPS) uhnsw_wsearch_kernel(const QueryArgs a) {
+  chain_begin(a);
   if constexpr (SLOTS == kWarpSlotsMost || CPL == 3) {
     wsearch_block<T, TEAM, CPL, U, WARPS>(a, a.lay);
   } else {
     const SmemLayout L(a.d_pad, a.ef_cap, a.hash_bits, a.cmax, a.k_max, 0, a.stage_bytes);
     wsearch_block<T, TEAM, CPL, U, WARPS>(a, L);
   }
+  chain_end(a);
 }
 
 }  // namespace uhnsw_dev

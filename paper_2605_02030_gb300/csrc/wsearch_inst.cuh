@@ -22,10 +22,7 @@ auto wsearch_kernel(bool most) {
 template <typename T, int TEAM, int CPL, int U>
 cudaError_t wlaunch_one(bool most, const QueryArgs& a, int grid, size_t smem, cudaStream_t st) {
   auto kern = wsearch_kernel<T, TEAM, CPL, U>(most);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  kern<<<grid, kWarpsPerBlock * 32, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_search_kernel(kern, grid, kWarpsPerBlock * 32, smem, a, st);
 }
 
 template <typename T, int TEAM, int CPL, int U>
