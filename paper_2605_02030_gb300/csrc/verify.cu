@@ -16,20 +16,24 @@ cudaError_t launch_verify_warps(const QueryArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// Warps per query, us for queries x candidates (128 dimensions, 152 SMs; the
-// last column 960 dimensions; K = 50 for 300 candidates, else 10):
-//               1 x 300  456 x 300  1,000 x 300  5,003 x 300  10,000 x 64  10,000 x 10  2,500 x 64
-//   8 warps          43         50           80          223          225          152         160
-//   4 warps          49         56           83          199          132           96         140
-//   2 warps          66         70           80          215          125           76         155
-// Eight while all queries are resident at once (3 blocks of 9 warps an SM):
-// the steps of one query are then what takes the time.  Two where one step of
-// two warps covers the list, as more warps would find no rows to sum, and for
-// up to 64 short rows: in steps of 32 or 64 none of them would be dropped.
+// Warps per query, us of back-to-back calls of queries x candidates (128
+// dimensions, the last column 960; Algorithm 1 with K = 10):
+//               1 x 300   456 x 300   3,000 x 200   3,000 x 500   10,000 x 90   3,000 x 500   3,000 x 24
+//                 exact       exact         exact         exact         exact   Algorithm 1  Algorithm 1
+//   8 warps          43          50            99           169           214            78          240
+//   4 warps          49          56            79           159           123            49          142
+//   2 warps          66          70            75           166           119            38           93
+// Eight while all queries are resident at once (3 blocks of 9 warps an SM): the
+// steps of one query are then what takes the time.  Past that, two for up to
+// 256 candidates between two barriers of Algorithm 1 (the exact mode has
+// none): more warps find few rows to sum.  Two as well for up to 64 short
+// rows: in steps of 32 or 64 none of them would be dropped.
 cudaError_t launch_verify(const QueryArgs& a, int num_sms, cudaStream_t st) {
-  if (a.cand_t <= (a.d_pad <= 256 ? 64 : 16)) return launch_verify_warps<2>(a, st);
+  if (a.cand_t <= 64 && a.d_pad <= 256) return launch_verify_warps<2>(a, st);
   if (a.nq <= 3 * (int64_t)num_sms) return launch_verify_warps<8>(a, st);
-  return launch_verify_warps<4>(a, st);
+  int span = a.cand_t;
+  if (a.mode == UHNSW_VERIFY_PAPER) span = a.kappa > a.k_max ? a.kappa : a.k_max;
+  return span <= 256 ? launch_verify_warps<2>(a, st) : launch_verify_warps<4>(a, st);
 }
 
 // FP32 master rows -> FP16 / BF16 traversal rows (round to nearest even).
