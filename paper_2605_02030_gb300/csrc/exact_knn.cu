@@ -25,6 +25,7 @@
 // ends once no query is left: sums never decrease, so no answer changes.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <climits>
 
 #include "coop_kernels.cuh"
@@ -323,19 +324,27 @@ __global__ void exact_merge_kernel(const unsigned long long* part, int nslices, 
 }
 
 namespace {
-// Warps of a block that take different queries: 16, 8 or 4 queries per block.
-int exact_wq(int64_t nq) { return nq > 8 ? 4 : nq > 4 ? 2 : 1; }
+// Warps of a block that take different queries: 16, 8 or 4 queries per block;
+// fewer where the tiles of so few rows would not give each of 152 SMs two blocks
+// (1,089 x 134, 144 queries: 74 -> 44 us; 1,083 x 146, 57 queries: 82 -> 61).
+int exact_wq(int64_t n, int64_t nq) {
+  const int64_t tiles = (n + kExTR - 1) / kExTR;
+  int wq = nq > 8 ? 4 : nq > 4 ? 2 : 1;
+  while (wq > 1 && tiles * ((nq + wq * kExQW - 1) / (wq * kExQW)) < 304) wq /= 2;
+  return wq;
+}
 }  // namespace
 
 int exact_workspace_slices(int64_t n, int64_t nq, int k, int num_sms) {
-  const int wq = exact_wq(nq);
+  const int wq = exact_wq(n, nq);
   const int64_t qb = (nq + wq * kExQW - 1) / (wq * kExQW);
   const int64_t slots = (int64_t)(wq == 4 ? kExPerSm<4> : kExPerSm<1>) * num_sms;
   // as many blocks along the rows as fill whole rounds of the GPU best; more
   // rounds only where fewer leave over 4 % of it idle
+  const int64_t cap = std::max<int64_t>(1, std::min<int64_t>(8192 / k, (n + kExTR - 1) / kExTR));
   int64_t best = 1;
   double fill = 0.0;
-  for (int64_t s = 1; s * qb <= 8 * slots || s == 1; ++s) {
+  for (int64_t s = 1; s <= cap && (s * qb <= 8 * slots || s == 1); ++s) {
     const int64_t blocks = s * qb, rounds = (blocks + slots - 1) / slots;
     const double f = (double)blocks / (double)(rounds * slots);
     if (f > fill + 0.04) {
@@ -344,11 +353,7 @@ int exact_workspace_slices(int64_t n, int64_t nq, int k, int num_sms) {
     }
     if (s >= slots) break;
   }
-  int64_t s = best;
-  const int64_t cap = 8192 / k;
-  if (s > cap) s = cap;
-  if (s > (n + kExTR - 1) / kExTR) s = (n + kExTR - 1) / kExTR;
-  return (int)(s < 1 ? 1 : s);
+  return (int)best;
 }
 
 template <int WQ>
@@ -370,7 +375,7 @@ cudaError_t launch_exact(const float* base, int64_t n, int d, int d_pad, const f
                          const float* p, int64_t nq, int k, int nslices, void* ws,
                          int64_t* out_ids, float* out_dist, cudaStream_t st) {
   unsigned long long* part = static_cast<unsigned long long*>(ws);
-  const int wq = exact_wq(nq);
+  const int wq = exact_wq(n, nq);
   cudaError_t e = wq == 4   ? launch_slices<4>(base, n, d, d_pad, q, p, nq, k, nslices, part, st)
                   : wq == 2 ? launch_slices<2>(base, n, d, d_pad, q, p, nq, k, nslices, part, st)
                             : launch_slices<1>(base, n, d, d_pad, q, p, nq, k, nslices, part, st);
