@@ -732,7 +732,7 @@ __device__ void coop_query(const QueryArgs& a, int64_t qi, unsigned char* smem,
   const float tau = query_tau(a, qi);
   int tn = 0, np = 0, terms = 0;
   for (int i = 0; i < nc;) {
-    const int bend = !paper ? nc : i == 0 ? min(k, nc) : min(i + kappa, nc);
+    const int bend = !paper ? nc : i == 0 ? min(k, nc) : i + min(kappa, nc - i);  // (kappa may be INT_MAX)
     const bool batch = i > 0;
     if (batch) {
       for (int j = tid; j < tn; j += THREADS) top[j] |= 1ull;  // mark R

@@ -415,7 +415,7 @@ __device__ __forceinline__ void warp_verify_run(const QueryArgs& a, const float*
   const bool paper = !exact && a.mode == UHNSW_VERIFY_PAPER;
   const int n0 = paper ? min(k, t) : t;
   for (int i = 0; i < t;) {
-    const int bend = i == 0 ? n0 : min(i + kappa, t);
+    const int bend = i == 0 ? n0 : i + min(kappa, t - i);  // (kappa may be INT_MAX)
     if (i > 0) {
       for (int j = lane; j < v.tn; j += 32) v.ci_()[j] |= kExpanded;  // mark R
       __syncwarp();
