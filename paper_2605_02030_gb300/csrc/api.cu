@@ -996,12 +996,15 @@ extern "C" int uhnsw_idealized_recall(uhnsw_index* idx, const float* q, const fl
   if (nq > 0 && (!q || !p || !counts)) return fail(UHNSW_EINVAL, "uhnsw_idealized_recall: NULL pointer");
   if (nq == 0) return UHNSW_OK;
   const float cut = cutoff > 0.f ? cutoff : 1.4f;
-  const int ns = std::max(exact_workspace_slices(idx->n, nq, K, idx->num_sms),
-                          exact_workspace_slices(idx->n, nq, t_max, idx->num_sms));
+  // each search has its own number of slices: a slice's list holds k keys, and the
+  // merge takes at most kExactMergeKeys of them
+  const int ns_k = exact_workspace_slices(idx->n, nq, K, idx->num_sms);
+  const int ns_t = exact_workspace_slices(idx->n, nq, t_max, idx->num_sms);
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   const size_t b_ik = (size_t)nq * K * 8, b_dk = (size_t)nq * K * 4;
   const size_t b_it = (size_t)nq * t_max * 8, b_dt = (size_t)nq * t_max * 4;
-  const size_t b_pb = (size_t)nq * 4, b_ws = (size_t)ns * nq * t_max * 8;
+  const size_t b_pb = (size_t)nq * 4;
+  const size_t b_ws = (size_t)std::max((int64_t)ns_k * K, (int64_t)ns_t * t_max) * nq * 8;
   const size_t need = al(b_ik) + al(b_dk) + al(b_it) + al(b_dt) + al(b_pb) + al(b_ws);
   char* buf = nullptr;
   cudaError_t e = cudaMalloc(&buf, need);
@@ -1016,10 +1019,11 @@ extern "C" int uhnsw_idealized_recall(uhnsw_index* idx, const float* q, const fl
   cudaStream_t st = (cudaStream_t)stream;
   const float gp0 = idx->gp[0], gp1 = idx->gp[1];
   // exact L_p top-K, exact base-metric top-t_max, then the curves
-  e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, p, nq, K, ns, ws, ik, dk, st);
+  e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, p, nq, K, ns_k, ws, ik, dk, st);
   if (e == cudaSuccess) e = launch_base_p(p, nq, gp0, gp1, cut, pb, st);
   if (e == cudaSuccess)
-    e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, pb, nq, t_max, ns, ws, it, dt, st);
+    e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, pb, nq, t_max, ns_t, ws, it,
+                     dt, st);
   if (e == cudaSuccess) e = launch_recall_curve(ik, it, nq, K, t_max, counts, st);
   cudaError_t e2 = cudaStreamSynchronize(st);
   cudaFree(buf);

@@ -341,7 +341,8 @@ int exact_workspace_slices(int64_t n, int64_t nq, int k, int num_sms) {
   const int64_t slots = (int64_t)(wq == 4 ? kExPerSm<4> : kExPerSm<1>) * num_sms;
   // as many blocks along the rows as fill whole rounds of the GPU best; more
   // rounds only where fewer leave over 4 % of it idle
-  const int64_t cap = std::max<int64_t>(1, std::min<int64_t>(8192 / k, (n + kExTR - 1) / kExTR));
+  const int64_t tiles = (n + kExTR - 1) / kExTR;
+  const int64_t cap = std::max<int64_t>(1, std::min<int64_t>(kExactMergeKeys / k, tiles));
   int64_t best = 1;
   double fill = 0.0;
   for (int64_t s = 1; s <= cap && (s * qb <= 8 * slots || s == 1); ++s) {
@@ -374,6 +375,7 @@ static cudaError_t launch_slices(const float* base, int64_t n, int d, int d_pad,
 cudaError_t launch_exact(const float* base, int64_t n, int d, int d_pad, const float* q,
                          const float* p, int64_t nq, int k, int nslices, void* ws,
                          int64_t* out_ids, float* out_dist, cudaStream_t st) {
+  if (nslices < 1 || nslices * (int64_t)k > kExactMergeKeys) return cudaErrorInvalidValue;
   unsigned long long* part = static_cast<unsigned long long*>(ws);
   const int wq = exact_wq(n, nq);
   cudaError_t e = wq == 4   ? launch_slices<4>(base, n, d, d_pad, q, p, nq, k, nslices, part, st)

@@ -89,7 +89,10 @@ cudaError_t launch_base_p(const float* p, int64_t nq, float gp0, float gp1, floa
                           float* out, cudaStream_t st);
 cudaError_t launch_recall_curve(const int64_t* ids_k, const int64_t* ids_t, int64_t nq, int K,
                                 int T, int32_t* counts, cudaStream_t st);
-// Exhaustive search: ws holds nslices x nq x k 8-byte keys.
+// Exhaustive search: ws holds nslices x nq x k 8-byte keys.  nslices is at most
+// exact_workspace_slices of the same k; more than kExactMergeKeys / k are refused
+// (cudaErrorInvalidValue): the merge holds a query's keys in shared memory.
+constexpr int kExactMergeKeys = 8192;
 int exact_workspace_slices(int64_t n, int64_t nq, int k, int num_sms);
 cudaError_t launch_exact(const float* base, int64_t n, int d, int d_pad, const float* q,
                          const float* p, int64_t nq, int k, int nslices, void* ws,
