@@ -651,6 +651,15 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
     return 0;
   };
 
+  // The warp kernel's 32-warp form: each query runs slower, so it is taken where 24
+  // warps per SM would leave queries for one more round, or for over two rounds.
+  // 32 against 24 warps, FP32 rows at ef 40 to 100 (40k x 50, 200k x 32, 1M x 128):
+  // 1.00 to 1.09 times the time at 1,800 to 3,600 queries, 0.75 to 1.00 at 4,500,
+  // 0.91 to 1.09 at 6,000, 0.94 to 1.03 at 10,000.
+  const bool most_pays = (nq > (int64_t)kWarpSlots * idx->num_sms &&
+                          nq <= (int64_t)kWarpSlotsMost * idx->num_sms) ||
+                         nq > 2 * (int64_t)kWarpSlots * idx->num_sms;
+
   // One launch description for a beam bound: kernel kind, layout, grid.
   auto describe = [&](int bound, Launch* Lo) -> int {
     Lo->a = a;
@@ -668,8 +677,10 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
       const size_t smem = (size_t)Lw.total * kWarpsPerBlock;
       if (4 * (size_t)Lw.total <= kSmemMax) {  // (a limit of the interface, as four per block)
         Lo->shape = wsh;
-        // (the 1 KB that a block reserves beside its own counts too)
-        Lo->shape.most = kSmSmem / (smem + 1024) * kWarpsPerBlock >= (size_t)kWarpSlotsMost;
+        // 32 warps per SM where shared memory holds them (the 1 KB that a block
+        // reserves beside its own counts too) and they save a round of queries
+        Lo->shape.most = kSmSmem / (smem + 1024) * kWarpsPerBlock >= (size_t)kWarpSlotsMost &&
+                         most_pays;
         Lo->smem = smem;
         Lo->a.cmax = cmax;
         Lo->a.stage_bytes = sv * vrow;
@@ -677,7 +688,7 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
         Lo->a.sv = sv;
         Lo->grid = (int)((nq + kWarpsPerBlock - 1) / kWarpsPerBlock);
         if (P->persistent) {
-          const int occ = wsearch_occupancy(idx->tdtype, wsh, smem);
+          const int occ = wsearch_occupancy(idx->tdtype, Lo->shape, smem);
           if (occ < 1) return fail(UHNSW_ECUDA, "uhnsw_search: kernel does not fit (smem %zu)", smem);
           Lo->grid = (int)std::min<int64_t>(Lo->grid, (int64_t)occ * idx->num_sms);
         }
