@@ -607,11 +607,12 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
   // steps, and more warps shorten it (1M x 128 FP16, ef 64, one query: 8 warps
   // 85 us, 4 warps 99, 2 warps 104, the warp kernel 194).  Queries that cannot
   // all be resident: `fallback` warps, or no (false) for 0.
-  auto describe_coop = [&](int bound, const WarpShape& sh, int fallback, Launch* Lo) -> bool {
+  auto describe_coop = [&](int bound, WarpShape sh, int fallback, Launch* Lo) -> bool {
     const int64_t per_sm = (nq + idx->num_sms - 1) / idx->num_sms;
     for (int i = kCoopForms - 1; i >= -1; --i) {
       const int nw = i >= 0 ? kCoopWarps[i] : fallback;
       if (nw == 0) return false;
+      sh.most = i < 0 && nw == kCoopManyWarps;
       const int cmax = (std::max(width * deg0, deg) + nw - 1) / nw * nw;
       const int ext = sh.team * sh.cpl * (idx->tdtype == UHNSW_F32 ? 4 : 8);
       int hb = Lo->a.hash_bits;
@@ -637,17 +638,31 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
     return false;
   };
 
-  // Distance warps per query of a launch whose queries are not all resident (0:
-  // the warp kernel).  Measured against the warp kernel, 2 warps per query:
-  //   rows above 64 chunks (960 BF16, 1,023 FP32): 0.98 to 1.99 times its
-  //     speed at 1,500 to 10,000 queries, ef 52 to 300;
+  // Distance warps per query of a cooperative launch whose queries are not all
+  // resident (the measurements are at kCoopManyWarps): four for rows above 64
+  // chunks and for FP32 rows above 32, two for shorter ones (400k x 500 FP16, ef
+  // 64: 5.1 ms with two and 5.8 with four; 1M x 128 FP16 2.9 and 3.2) and for FP32
+  // rows of 16 chunks a lane (50k x 2,000: 15.6 and 16.4).
+  auto coop_warps = [&](const WarpShape& sh) -> int {
+    const int row = sh.team * sh.cpl;
+    return sh.cpl <= 8 && (row > 64 || (row > 32 && idx->tdtype == UHNSW_F32)) ? kCoopManyWarps : 2;
+  };
+
+  // The same, where the warp kernel could take the launch (0: it does).  The
+  // cooperative kernel's speed against the warp kernel's:
+  //   rows above 64 chunks: 1.00 to 2.6 times at ef 64 and 128 (16-bit rows of 600
+  //     to 1,500 dimensions, FP32 rows of 500 to 1,500; 3,300 to 10,000 queries);
+  //   but FP32 rows that leave a fifth of a team's 128 chunks empty (300 and 400
+  //     dimensions): 0.77 and 0.82 at 10,000 queries of ef 64, 1.03 to 1.25 at ef 128
+  //     and 300 and, at ef 64, with 1,300 queries;
   //   33 to 64 chunks (500 FP16, 200 and 500 FP32): 1.04 to 2.4 at ef 300;
   //     at ef 52 and 64, 1.15 to 1.75 up to 2,500 queries, 0.67 to 1.28 above;
   //   narrower rows: 0.7 to 1.4 at 1,500 queries, 0.6 to 0.9 at 10,000.
   auto coop_anyway = [&](const WarpShape& sh, int bound) -> int {
     const int row = sh.team * sh.cpl;
-    if (row > 64) return 2;
-    if (row > 32 && (bound > 128 || nq <= 20 * (int64_t)idx->num_sms)) return 2;
+    const bool thin = idx->tdtype == UHNSW_F32 && row == 128 && 5 * chunks <= 4 * row;
+    if (row > 64 && !thin) return coop_warps(sh);
+    if (row > 32 && (bound > 128 || nq <= 20 * (int64_t)idx->num_sms)) return coop_warps(sh);
     return 0;
   };
 
@@ -698,7 +713,7 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
         return fail(UHNSW_ECAPACITY, "uhnsw_search: %zu bytes of shared memory per block", smem);
     }
     // the block-per-query form: one query per block
-    if (describe_coop(bound, bsh, 2, Lo)) return UHNSW_OK;
+    if (describe_coop(bound, bsh, coop_warps(bsh), Lo)) return UHNSW_OK;
     return fail(UHNSW_ECAPACITY, "uhnsw_search: no launch fits");
   };
 

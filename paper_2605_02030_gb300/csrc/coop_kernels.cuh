@@ -785,9 +785,10 @@ __device__ void coop_query(const QueryArgs& a, int64_t qi, unsigned char* smem,
   }
 }
 
-// Blocks per SM asked of the register allocator.  Eight distance warps serve
-// launches of at most one block per SM and take the registers they want: at
-// 72 registers (3 blocks) the spills cost 2,403 against 1,779 cycles a merge.
+// Blocks per SM asked of the register allocator where all queries are resident.
+// Eight distance warps serve launches of at most one block per SM and take the
+// registers they want: at 72 registers (3 blocks) the spills cost 2,403 against
+// 1,779 cycles a merge.
 template <int CPL, int NW>
 struct CoopMinBlocks {
   static constexpr int value = NW >= 8    ? 1
@@ -797,9 +798,33 @@ struct CoopMinBlocks {
                                           : 3;
 };
 
+// The form for more queries than are resident, of rows whose sums are what a step
+// takes: four distance warps and a block more per SM.  A resident query is slower
+// in it (300 to 600 queries of 1M x 128 and 400k x 500 FP16, ef 64: 1.05 to 1.18
+// times the time), so that those keep CoopMinBlocks.  10,000 queries, ms; this
+// form, two distance warps, and the kernel they replaced (four warps per query, each
+// summing and merging in turn):
+//   1M x 960 BF16, ef 512, k 100                          90.4, 108.5, 101.5
+//   the same rows, mixed k and ef, one launch             37.4, 44.8, 48.2
+//   the same, launches queued on two streams              38.3, 45.8, 37.9
+//   200k x 960 FP16, ef 64 and 300                        6.5, 7.7, 10.8; 19.5, 20.0, 37.4
+//   200k x 960 FP32                                       11.3, 16.1, 14.6; 27.9, 36.0, 45.5
+//   200k x 200 FP32                                       4.1, 4.4, 3.6; 19.9, 21.9, 17.9
+// Four warps at CoopMinBlocks' four blocks took 100.9 ms for the first row, eight
+// 129.8; two warps at seven blocks 118.8.  FP32 rows of four chunks a lane would
+// spill at five blocks and take four warps at four (200k x 400, ef 64: 5.9 ms, 6.3
+// with spills, 6.8 with two warps).
+constexpr int kCoopManyWarps = 4;
+template <typename T, int TEAM, int CPL>
+constexpr bool coop_has_many() {
+  return TEAM == 32 && (CPL == 8 || CPL == (std::is_same<T, float>::value ? 2 : 4));
+}
+template <int CPL>
+constexpr int kCoopManyBlocks = CPL <= 4 ? 5 : 4;
+
 // One block of NW + 1 warps per query; a.queue_head set = persistent.
-template <typename T, int TEAM, int CPL, int U, int NW>
-__global__ void __launch_bounds__((NW + 1) * 32, (CoopMinBlocks<CPL, NW>::value))
+template <typename T, int TEAM, int CPL, int U, int NW, int BLOCKS>
+__global__ void __launch_bounds__((NW + 1) * 32, BLOCKS)
     uhnsw_csearch_kernel(const QueryArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int next;

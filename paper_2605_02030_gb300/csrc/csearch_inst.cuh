@@ -15,18 +15,26 @@ struct CoopRows {
 };
 
 template <typename T, int TEAM, int CPL, int NW>
-cudaError_t claunch_one(const QueryArgs& a, int grid, size_t smem, cudaStream_t st) {
-  auto kern = uhnsw_csearch_kernel<T, TEAM, CPL, CoopRows<CPL>::value, NW>;
-  return launch_search_kernel(kern, grid, (NW + 1) * 32, smem, a, st);
+auto csearch_kernel(bool most) {
+  constexpr int U = CoopRows<CPL>::value;
+  auto kern = uhnsw_csearch_kernel<T, TEAM, CPL, U, NW, CoopMinBlocks<CPL, NW>::value>;
+  if constexpr (NW == kCoopManyWarps && coop_has_many<T, TEAM, CPL>())
+    if (most) kern = uhnsw_csearch_kernel<T, TEAM, CPL, U, NW, kCoopManyBlocks<CPL>>;
+  return kern;
+}
+
+template <typename T, int TEAM, int CPL, int NW>
+cudaError_t claunch_one(bool most, const QueryArgs& a, int grid, size_t smem, cudaStream_t st) {
+  return launch_search_kernel(csearch_kernel<T, TEAM, CPL, NW>(most), grid, (NW + 1) * 32, smem, a, st);
 }
 
 // Resident blocks per SM that the registers allow (0: the query failed).
-template <typename T, int TEAM, int CPL, int NW>
+template <typename T, int TEAM, int CPL, int NW, bool MOST>
 int cregs_one() {
   static const int blocks = [] {
     int nb = 0;
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &nb, uhnsw_csearch_kernel<T, TEAM, CPL, CoopRows<CPL>::value, NW>, (NW + 1) * 32, 0);
+        &nb, csearch_kernel<T, TEAM, CPL, NW>(MOST), (NW + 1) * 32, 0);
     return e == cudaSuccess ? nb : 0;
   }();
   return blocks;
@@ -55,8 +63,9 @@ int cregs_one() {
     }                                                               \
   } while (0)
 
-#define CLAUNCH_CALL(T, TEAM, CPL, NW) claunch_one<T, TEAM, CPL, NW>(a, grid, smem, st)
-#define CREGS_CALL(T, TEAM, CPL, NW) cregs_one<T, TEAM, CPL, NW>()
+#define CLAUNCH_CALL(T, TEAM, CPL, NW) claunch_one<T, TEAM, CPL, NW>(sh.most, a, grid, smem, st)
+#define CREGS_CALL(T, TEAM, CPL, NW) \
+  (sh.most ? cregs_one<T, TEAM, CPL, NW, true>() : cregs_one<T, TEAM, CPL, NW, false>())
 
 template <typename T, int NW>
 cudaError_t claunch_shape(WarpShape sh, const QueryArgs& a, int grid, size_t smem, cudaStream_t st) {
