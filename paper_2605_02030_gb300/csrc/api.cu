@@ -1003,7 +1003,7 @@ extern "C" int uhnsw_exact(uhnsw_index* idx, const float* q, const float* p, int
     idx->exact_ws_bytes = need;
   }
   cudaError_t e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, p, nq, k, ns,
-                               idx->exact_ws, out_ids, out_dist, (cudaStream_t)stream);
+                               idx->num_sms, idx->exact_ws, out_ids, out_dist, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "uhnsw_exact: launch");
   return UHNSW_OK;
 }
@@ -1045,11 +1045,12 @@ extern "C" int uhnsw_idealized_recall(uhnsw_index* idx, const float* q, const fl
   cudaStream_t st = (cudaStream_t)stream;
   const float gp0 = idx->gp[0], gp1 = idx->gp[1];
   // exact L_p top-K, exact base-metric top-t_max, then the curves
-  e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, p, nq, K, ns_k, ws, ik, dk, st);
+  e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, p, nq, K, ns_k, idx->num_sms, ws, ik,
+                   dk, st);
   if (e == cudaSuccess) e = launch_base_p(p, nq, gp0, gp1, cut, pb, st);
   if (e == cudaSuccess)
-    e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, pb, nq, t_max, ns_t, ws, it,
-                     dt, st);
+    e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, pb, nq, t_max, ns_t, idx->num_sms,
+                     ws, it, dt, st);
   if (e == cudaSuccess) e = launch_recall_curve(ik, it, nq, K, t_max, counts, st);
   cudaError_t e2 = cudaStreamSynchronize(st);
   cudaFree(buf);
@@ -1135,8 +1136,8 @@ extern "C" int uhnsw_exact_static(uhnsw_index* idx, const float* q, const float*
   int ns = exact_workspace_slices(idx->n, nq, k, idx->num_sms);
   const int64_t fit = (int64_t)UHNSW_EXACT_STATIC_BYTES / per_slice;
   if (ns > fit) ns = (int)fit;
-  e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, p, nq, k, ns, base, out_ids,
-                   out_dist, (cudaStream_t)stream);
+  e = launch_exact(idx->base32, idx->n, idx->d, idx->d_pad, q, p, nq, k, ns, idx->num_sms,
+                   base, out_ids, out_dist, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "uhnsw_exact_static: launch");
   return UHNSW_OK;
 }

@@ -249,16 +249,18 @@ __global__ void __launch_bounds__(kExBlock, kExPerSm<WQ>) exact_slice_kernel(
     }
   }
   if (GROUPS > 1) {
-    // the other groups' lists into the first group's
+    // the groups' lists of a query into one of them: each group takes its share of
+    // the queries (1,000 x 8, 60 queries, k 1: 33 us by the first group alone, 21 now)
     __shared__ int gn[kExWarps][kExQW];
 #pragma unroll
     for (int u = 0; u < kExQW; ++u)
       if (lane == 0) gn[warp][u] = tn[u];
     __syncthreads();
-    if (group > 0) return;
 #pragma unroll
-    for (int u = 0; u < kExQW; ++u)
-      for (int w = warp + WQ; w < kExWarps; w += WQ) {
+    for (int u = 0; u < kExQW; ++u) {
+      if (u % GROUPS != group) continue;
+      for (int w = wq; w < kExWarps; w += WQ) {
+        if (w == warp) continue;
         const unsigned long long* other =
             reinterpret_cast<unsigned long long*>(smem + L.top) + (w * kExQW + u) * k;
         for (int e = 0; e < gn[w][u]; e += kExTR) {
@@ -268,11 +270,12 @@ __global__ void __launch_bounds__(kExBlock, kExPerSm<WQ>) exact_slice_kernel(
           __syncwarp();
         }
       }
+    }
   }
 #pragma unroll
   for (int u = 0; u < kExQW; ++u) {
     const int64_t qi = q0 + wq * kExQW + u;
-    if (qi >= nq) continue;
+    if (qi >= nq || u % GROUPS != group) continue;
     for (int j = lane; j < k; j += 32)
       part[(slice * nq + qi) * k + j] = j < tn[u] ? top[u * k + j] : kNoKey;
   }
@@ -324,29 +327,39 @@ __global__ void exact_merge_kernel(const unsigned long long* part, int nslices, 
 }
 
 namespace {
-// Warps of a block that take different queries: 16, 8 or 4 queries per block;
-// fewer where the tiles of so few rows would not give each of 152 SMs two blocks
+// Warps of a block that take different queries: 16, 8 or 4 queries per block.
+// Eight for lists of up to 128 where one tile at a time would give an SM less
+// than 14 blocks of 16 (a warp's merges, four queries one after the other, are then
+// what takes the time): 3,000 x 32, 250 queries, k 10: 48 us with eight and 75 with
+// sixteen; 1,000 x 8, 4,000 queries, k 32: 126, 148; 1,165 x 16, 2,139 queries, k
+// 10: 78, 101; past it 1,500 x 60, 3,000 queries: 215, 188; k 256 on 1,000 x 8, 600
+// queries: 192, 173.  Four where two blocks an SM are not reached otherwise
 // (1,089 x 134, 144 queries: 74 -> 44 us; 1,083 x 146, 57 queries: 82 -> 61).
-int exact_wq(int64_t n, int64_t nq) {
+int exact_wq(int64_t n, int64_t nq, int k, int num_sms) {
   const int64_t tiles = (n + kExTR - 1) / kExTR;
+  auto blocks = [&](int wq) { return tiles * ((nq + wq * kExQW - 1) / (wq * kExQW)); };
   int wq = nq > 8 ? 4 : nq > 4 ? 2 : 1;
-  while (wq > 1 && tiles * ((nq + wq * kExQW - 1) / (wq * kExQW)) < 304) wq /= 2;
+  if (wq == 4 && blocks(4) < (k <= 128 ? 14 : 2) * (int64_t)num_sms) wq = 2;
+  if (wq == 2 && blocks(2) < 2 * (int64_t)num_sms) wq = 1;
   return wq;
 }
 }  // namespace
 
 int exact_workspace_slices(int64_t n, int64_t nq, int k, int num_sms) {
-  const int wq = exact_wq(n, nq);
+  const int wq = exact_wq(n, nq, k, num_sms);
   const int64_t qb = (nq + wq * kExQW - 1) / (wq * kExQW);
   const int64_t slots = (int64_t)(wq == 4 ? kExPerSm<4> : kExPerSm<1>) * num_sms;
   // as many blocks along the rows as fill whole rounds of the GPU best; more
-  // rounds only where fewer leave over 4 % of it idle
+  // rounds only where fewer leave over 4 % of it idle and a slice keeps 16 tiles:
+  // every slice fills its own list, and the merge takes a list per slice (3,000 x
+  // 32, 2,500 queries: k 10 4 slices 198 us, 19 slices 284; k 200 818 and 2,521)
   const int64_t tiles = (n + kExTR - 1) / kExTR;
   const int64_t cap = std::max<int64_t>(1, std::min<int64_t>(kExactMergeKeys / k, tiles));
   int64_t best = 1;
   double fill = 0.0;
   for (int64_t s = 1; s <= cap && (s * qb <= 8 * slots || s == 1); ++s) {
     const int64_t blocks = s * qb, rounds = (blocks + slots - 1) / slots;
+    if (s > 1 && rounds > 1 && (tiles + s - 1) / s < 16) break;
     const double f = (double)blocks / (double)(rounds * slots);
     if (f > fill + 0.04) {
       best = s;
@@ -373,11 +386,11 @@ static cudaError_t launch_slices(const float* base, int64_t n, int d, int d_pad,
 }
 
 cudaError_t launch_exact(const float* base, int64_t n, int d, int d_pad, const float* q,
-                         const float* p, int64_t nq, int k, int nslices, void* ws,
+                         const float* p, int64_t nq, int k, int nslices, int num_sms, void* ws,
                          int64_t* out_ids, float* out_dist, cudaStream_t st) {
   if (nslices < 1 || nslices * (int64_t)k > kExactMergeKeys) return cudaErrorInvalidValue;
   unsigned long long* part = static_cast<unsigned long long*>(ws);
-  const int wq = exact_wq(n, nq);
+  const int wq = exact_wq(n, nq, k, num_sms);
   cudaError_t e = wq == 4   ? launch_slices<4>(base, n, d, d_pad, q, p, nq, k, nslices, part, st)
                   : wq == 2 ? launch_slices<2>(base, n, d, d_pad, q, p, nq, k, nslices, part, st)
                             : launch_slices<1>(base, n, d, d_pad, q, p, nq, k, nslices, part, st);

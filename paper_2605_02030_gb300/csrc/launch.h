@@ -96,7 +96,7 @@ cudaError_t launch_recall_curve(const int64_t* ids_k, const int64_t* ids_t, int6
 constexpr int kExactMergeKeys = 8192;
 int exact_workspace_slices(int64_t n, int64_t nq, int k, int num_sms);
 cudaError_t launch_exact(const float* base, int64_t n, int d, int d_pad, const float* q,
-                         const float* p, int64_t nq, int k, int nslices, void* ws,
+                         const float* p, int64_t nq, int k, int nslices, int num_sms, void* ws,
                          int64_t* out_ids, float* out_dist, cudaStream_t st);
 
 // per-storage-type entry points (defined in wsearch_<type>.cu and csearch_<type>_w<warps>.cu)
