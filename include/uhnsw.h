@@ -368,7 +368,9 @@ int uhnsw_exact_static(uhnsw_index* idx, const float* q, const float* p, int64_t
  * q [nq][d], p [nq]; k and ef for all) with 1 warm-up and 3 timed launches on
  * `stream`, and records the fastest for the bucket (traversal dtype, beam
  * next_pow2(max(ef, k)), k next_pow2(k)) in the index; uhnsw_search with
- * opts->query_threads == 0 then uses it.  Candidates: the warp-per-query
+ * opts->query_threads == 0 then uses it (a choice of the warp kernel only where
+ * the queries are not all resident at once; the form for those that are takes
+ * the chosen team width).  Candidates: the warp-per-query
  * kernel with each compiled team width that covers a row (8, 16, 32 lanes),
  * 4, 8 or 16 staged verification rows, the default visited table or one
  * twice its size, and a drop test every 1, 2 or 4 verification groups; the

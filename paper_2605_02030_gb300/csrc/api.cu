@@ -513,6 +513,10 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
   // autotuned choice) a beam bucket whose warp-kernel layout does not fit in
   // shared memory runs the cooperative kernel instead
   const bool forced = opts.query_threads != 0;
+  // (the caller's choices, as the autotuned ones take their place below)
+  const bool automatic = !forced && opts.team_lanes == 0 && opts.stage_bytes == 0;
+  const int hash_asked = opts.hash_bits;
+  bool tuned = false;
   if (opts.query_threads == 0) {
     // the autotuned configuration of this bucket, if any
     const int64_t key = ((int64_t)(1 << next_pow2_bits(ef_cap)) << 16) | (1 << next_pow2_bits(k_max));
@@ -524,6 +528,7 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
         opts.stage_bytes = tv.second.stage_bytes;
         if (opts.hash_bits == 0) opts.hash_bits = tv.second.hash_bits;
         if (opts.verify_groups == 0) opts.verify_groups = tv.second.verify_groups;
+        tuned = true;
         break;
       }
   }
@@ -606,8 +611,9 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
   // resident at once: a launch that small is bound by each query's own chain of
   // steps, and more warps shorten it (1M x 128 FP16, ef 64, one query: 8 warps
   // 85 us, 4 warps 99, 2 warps 104, the warp kernel 194).  Queries that cannot
-  // all be resident: `fallback` warps, or no (false) for 0.
-  auto describe_coop = [&](int bound, WarpShape sh, int fallback, Launch* Lo) -> bool {
+  // all be resident: `fallback` warps, or no (false) for 0.  hash: the visited
+  // table asked for (0: the default, or a larger one).
+  auto describe_coop = [&](int bound, WarpShape sh, int fallback, int hash, Launch* Lo) -> bool {
     const int64_t per_sm = (nq + idx->num_sms - 1) / idx->num_sms;
     for (int i = kCoopForms - 1; i >= -1; --i) {
       const int nw = i >= 0 ? kCoopWarps[i] : fallback;
@@ -615,13 +621,13 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
       sh.most = i < 0 && nw == kCoopManyWarps;
       const int cmax = (std::max(width * deg0, deg) + nw - 1) / nw * nw;
       const int ext = sh.team * sh.cpl * (idx->tdtype == UHNSW_F32 ? 4 : 8);
-      int hb = Lo->a.hash_bits;
+      int hb = visited_bits(hash, bound, width, deg0);
       size_t smem = CoopLayout(ext, bound, hb, cmax, k_max, nw + 1).total;
       const int occ = csearch_occupancy(idx->tdtype, nw, sh, smem);
       if (occ < 1 || (i >= 0 && occ < per_sm)) continue;
       // a larger visited table re-evaluates fewer nodes; it takes the shared
       // memory that the resident queries leave
-      while (opts.hash_bits == 0 && hb < 14) {
+      while (hash == 0 && hb < 14) {
         const size_t more = CoopLayout(ext, bound, hb + 1, cmax, k_max, nw + 1).total;
         if (csearch_occupancy(idx->tdtype, nw, sh, more) < std::min<int64_t>(per_sm, occ)) break;
         ++hb;
@@ -681,9 +687,11 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
     Lo->a.ef_cap = bound;
     Lo->a.hash_bits = visited_bits(opts.hash_bits, bound, width, deg0);
     if (want_warp) {
-      // the caller's (or the autotuner's) kernel, team or staging is kept
-      if (opts.query_threads == 0 && opts.team_lanes == 0 && opts.stage_bytes == 0 &&
-          describe_coop(bound, wsh, coop_anyway(wsh, bound), Lo))
+      // The caller's kernel, team or staging is kept, and the autotuner's where the
+      // queries are not all resident: it was timed on another batch, and with the
+      // warp kernel one query of 1M x 128 FP16 takes 194 us, not 85.
+      if (automatic &&
+          describe_coop(bound, wsh, tuned ? 0 : coop_anyway(wsh, bound), hash_asked, Lo))
         return UHNSW_OK;
       const int cmax = std::max({width * deg0, deg, 4});
       const int sv = sv_asked > 0 ? sv_asked
@@ -713,7 +721,7 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
         return fail(UHNSW_ECAPACITY, "uhnsw_search: %zu bytes of shared memory per block", smem);
     }
     // the block-per-query form: one query per block
-    if (describe_coop(bound, bsh, coop_warps(bsh), Lo)) return UHNSW_OK;
+    if (describe_coop(bound, bsh, coop_warps(bsh), opts.hash_bits, Lo)) return UHNSW_OK;
     return fail(UHNSW_ECAPACITY, "uhnsw_search: no launch fits");
   };
 
