@@ -580,11 +580,11 @@ __device__ void coop_query(const QueryArgs& a, int64_t qi, unsigned char* smem,
             if (level > 1) {
               if (f < g.deg) vnext = adj[f - g.deg];
             } else if (f < g.deg0) {
-              vnext = g.ell0[(int64_t)key_id(curk) * g.deg0 + f];
+              vnext = g.ell0[chk_idx(key_id(curk), a.n, 5, a.err) * g.deg0 + f];
             }
           }
         }
-        const int32_t ur = v >= 0 ? g.up_row[v] : -1;
+        const int32_t ur = v >= 0 ? g.up_row[chk_idx(v, a.n, 3, a.err)] : -1;
         nf += sum_slots(b, v, false, ckbuf(ph));
         const unsigned val = __ballot_sync(kFull, v >= 0);
         if (v >= 0)
@@ -671,13 +671,13 @@ __device__ void coop_query(const QueryArgs& a, int64_t qi, unsigned char* smem,
         const uint32_t was = __shfl_sync(kFull, par_next, slot_par & 31);
         int32_t v = -1;
         if (lane < spw && slot_par < npar)
-          v = mine == was ? vnext : g.ell0[(int64_t)mine * g.deg0 + slot_link];
+          v = mine == was ? vnext : g.ell0[chk_idx(mine, a.n, 5, a.err) * g.deg0 + slot_link];
         // the parents after these, if no candidate of this step is nearer
         par_next = step > 0 && lane < a.width ? key_id(pub[ph].uk[nWp + lane]) : kIdMask;
         const uint32_t then = __shfl_sync(kFull, par_next, slot_par & 31);
         vnext = -1;
         if (lane < spw && slot_par < a.width && then != kIdMask)
-          vnext = g.ell0[(int64_t)then * g.deg0 + slot_link];
+          vnext = g.ell0[chk_idx(then, a.n, 5, a.err) * g.deg0 + slot_link];
         nf = sum_slots(0, v, true, out);
       } else {
         for (int b = 0; b < spw; b += 32) {
@@ -685,7 +685,9 @@ __device__ void coop_query(const QueryArgs& a, int64_t qi, unsigned char* smem,
           const bool in = b + lane < spw && f < npar * g.deg0;
           const int j = in ? f / g.deg0 : 0;
           const uint32_t mine = __shfl_sync(kFull, par, j);
-          nf += sum_slots(b, in ? g.ell0[(int64_t)mine * g.deg0 + (f - j * g.deg0)] : -1, true, out);
+          const int32_t v =
+              in ? g.ell0[chk_idx(mine, a.n, 5, a.err) * g.deg0 + (f - j * g.deg0)] : -1;
+          nf += sum_slots(b, v, true, out);
         }
       }
       if (lane == 0) fresh_of[(ph ^ 1) * NW + warp] = nf;

@@ -176,14 +176,14 @@ __device__ __forceinline__ int block_select(const BuildArgs& a, const unsigned l
       const uint32_t w = __shfl_sync(kFull, kept[c], j & 31);
       if (j >> 5 == c) v = w;
     }
-    return a.X + (int64_t)v * a.d_pad;
+    return a.X + chk_idx(v, a.n, 22, a.err) * a.d_pad;
   };
   int r = 0, ph = 0;
   for (int i0 = 0; i0 < nw && r < m; i0 += G) {
     const int i = i0 + warp;
     const unsigned long long x = i < nw ? W[i] : kNoKey;
     const float dc = key_dist(x);
-    const float* xc = a.X + (int64_t)(i < nw ? key_id(x) : 0) * a.d_pad;
+    const float* xc = a.X + chk_idx(i < nw ? key_id(x) : 0, a.n, 21, a.err) * a.d_pad;
     bool keep = i < nw;
     for (int j0 = 0; j0 < r && keep; j0 += 8) {
       const float* ra = kept_row(min(j0 + team, r - 1));
@@ -206,7 +206,7 @@ __device__ __forceinline__ int block_select(const BuildArgs& a, const unsigned l
       if (!mask || r >= m) break;
       bool still = (mask >> warp) & 1u;
       if (still) {
-        const float* xs = a.X + (int64_t)id * a.d_pad;
+        const float* xs = a.X + chk_idx(id, a.n, 22, a.err) * a.d_pad;
         float sa, sb;
         build_dist2_metric(a.metric, xs, xs, xc, a.d_pad, lt, a.bp, sa, sb);
         still = dc < sa;
@@ -282,8 +282,9 @@ __global__ void __launch_bounds__((NW + 1) * 32, (NW >= 8 ? 1 : NW >= 4 ? 4 : 7)
       const int ia = i0 + team, ib = ia + 4;
       const uint32_t da = wl[min(ia, nf - 1)], db = wl[min(ib, nf - 1)];
       float sa, sb;
-      build_dist2_metric(a.metric, a.X + (int64_t)da * a.d_pad, a.X + (int64_t)db * a.d_pad, qv,
-                         a.d_pad, lt, a.bp, sa, sb);
+      build_dist2_metric(a.metric, a.X + chk_idx(da, a.n, 20, a.err) * a.d_pad,
+                         a.X + chk_idx(db, a.n, 20, a.err) * a.d_pad, qv, a.d_pad, lt, a.bp, sa,
+                         sb);
       if (lt == 0 && ia < nf) o[ia] = make_key(sa, da);
       if (lt == 0 && ib < nf) o[ib] = make_key(sb, db);
     }
@@ -310,7 +311,11 @@ __global__ void __launch_bounds__((NW + 1) * 32, (NW >= 8 ? 1 : NW >= 4 ? 4 : 7)
   const int lu = a.lv[u];
   const int64_t max_steps = ((int64_t)top + 1) * (a.n + 16);
   int64_t step = 0;
-  for (int l = top; l > lu && step < max_steps; ++step) {
+  for (int l = top; l > lu; ++step) {
+    if (step >= max_steps) {  // (never: every step is nearer, or a level lower)
+      if (tid == 0) set_error(a.err, UHNSW_ECAPACITY);
+      break;
+    }
     ph ^= 1;
     if (!merger) expand((int32_t)key_id(curk), l, false, ckbuf(ph));
     __syncthreads();
