@@ -450,7 +450,9 @@ typedef struct {
   int32_t max_batch;     /* queries per launch; 0 => 1024 */
   int32_t streams;       /* batches in flight at once (one stream each); 0 => 4 */
   int64_t state_budget;  /* bytes of search state (beam, visited table, verification lists
-                            of every admitted, unfinished query) admitted at once;
+                            of every admitted, unfinished query, as the kernel that needs
+                            most holds them) admitted at once; a visited table that a
+                            launch enlarges into shared memory left free is not counted;
                             0 => 2 * max_batch queries at ef_max / k_max */
   int32_t k_max;         /* largest k accepted; 0 => 100 */
   int32_t ef_max;        /* largest ef accepted; 0 => 512 */

@@ -1156,7 +1156,6 @@ int64_t uhnsw_internal::query_state_bytes(const uhnsw_index* idx, int32_t ef, in
   uhnsw_search_opts opts;
   std::memset(&opts, 0, sizeof(opts));
   if (o) opts = *o;
-  const bool warp = opts.query_threads != kBlock;
   const int width = std::max(1, opts.search_width);
   int deg0 = 0, deg = 0;
   for (auto& G : idx->g)
@@ -1164,15 +1163,25 @@ int64_t uhnsw_internal::query_state_bytes(const uhnsw_index* idx, int32_t ef, in
       deg0 = std::max(deg0, G.deg0);
       deg = std::max(deg, G.deg);
     }
-  const int efp = std::max(ef, k);
-  const int cmax = std::max({width * deg0, deg, warp ? 4 : kBlock / 8});
+  const int efp = std::max(ef, k), links = std::max(width * deg0, deg);
   const int hb = visited_bits(opts.hash_bits, efp, width, deg0);
-  int stage = 0;
-  if (warp) {
+  const int vec = idx->tdtype == UHNSW_F32 ? 4 : 8, chunks = idx->d_pad / vec;
+  // the larger of the kernels that prepare_search may launch
+  const bool block = opts.query_threads == kBlock;
+  const bool automatic = opts.query_threads == 0 && opts.team_lanes == 0 && opts.stage_bytes == 0;
+  int most = 0;
+  if (!block) {
     const int vrow = idx->d_pad * 4;
-    stage = std::max(4, (opts.stage_bytes > 0 ? opts.stage_bytes / vrow : 4) & ~3) * vrow;
+    const int stage = std::max(4, (opts.stage_bytes > 0 ? opts.stage_bytes / vrow : 4) & ~3) * vrow;
+    most = SmemLayout(idx->d_pad, efp, hb, std::max(links, 4), k, 0, stage).total;
   }
-  return SmemLayout(idx->d_pad, efp, hb, cmax, k, 0, stage).total;
+  WarpShape sh{0, 0, 0};
+  if (block ? pick_block_shape(idx->tdtype, chunks, &sh)
+            : automatic && pick_warp_shape(idx->tdtype, chunks, 0, false, &sh))
+    for (int nw : kCoopWarps)
+      most = std::max(most, CoopLayout(sh.team * sh.cpl * vec, efp, hb, (links + nw - 1) / nw * nw,
+                                       k, nw + 1).total);
+  return most;
 }
 
 extern "C" int uhnsw_autotune(uhnsw_index* idx, const float* q, const float* p, int64_t nq,
