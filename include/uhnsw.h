@@ -371,7 +371,7 @@ int uhnsw_exact_static(uhnsw_index* idx, const float* q, const float* p, int64_t
  * opts->query_threads == 0 then uses it (a choice of the warp kernel only where
  * the queries are not all resident at once; the form for those that are takes
  * the chosen team width).  Candidates: the warp-per-query
- * kernel with each compiled team width that covers a row (8, 16, 32 lanes),
+ * kernel with each compiled team width that covers a row (4, 8, 16, 32 lanes),
  * 4, 8 or 16 staged verification rows, the default visited table or one
  * twice its size, and a drop test every 1, 2 or 4 verification groups; the
  * block-per-query kernel with either table size.  The candidates run the same algorithm in the same

@@ -1325,7 +1325,7 @@ extern "C" int uhnsw_autotune_load(uhnsw_index* idx, const char* path) {
                            &stage, &hb, &vg);
     if (got != 7 && got != 9) continue;
     if (dt != (int)idx->tdtype || d != idx->d) continue;
-    if ((qt != 32 && qt != kBlock) || (team != 0 && team != 8 && team != 16 && team != 32) ||
+    if ((qt != 32 && qt != kBlock) || (team != 0 && team != 4 && team != 8 && team != 16 && team != 32) ||
         stage < 0 || stage > 64 * 1024 || efb < 1 || kb < 1 || hb < 0 || hb > 15 || vg < 0 ||
         vg > 16)
       continue;
