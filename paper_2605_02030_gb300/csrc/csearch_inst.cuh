@@ -3,6 +3,8 @@
 // of the block-per-query form (pick_warp_shape, pick_block_shape).
 #pragma once
 
+#include <atomic>
+
 #include "coop_kernels.cuh"
 #include "launch.h"
 
@@ -28,15 +30,18 @@ cudaError_t claunch_one(bool most, const QueryArgs& a, int grid, size_t smem, cu
   return launch_search_kernel(csearch_kernel<T, TEAM, CPL, NW>(most), grid, (NW + 1) * 32, smem, a, st);
 }
 
-// Resident blocks per SM that the registers allow (0: the query failed).
+// Resident blocks per SM that the registers allow, asked of the runtime once (0: it
+// failed, as it does where the kernel's first load finds no device memory; the next
+// call asks again).
 template <typename T, int TEAM, int CPL, int NW, bool MOST>
 int cregs_one() {
-  static const int blocks = [] {
-    int nb = 0;
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &nb, csearch_kernel<T, TEAM, CPL, NW>(MOST), (NW + 1) * 32, 0);
-    return e == cudaSuccess ? nb : 0;
-  }();
+  static std::atomic<int> known{0};
+  int blocks = known.load(std::memory_order_relaxed);
+  if (blocks > 0) return blocks;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &blocks, csearch_kernel<T, TEAM, CPL, NW>(MOST), (NW + 1) * 32, 0) != cudaSuccess)
+    return 0;
+  known.store(blocks, std::memory_order_relaxed);
   return blocks;
 }
 
