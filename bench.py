@@ -1500,8 +1500,8 @@ def run_profile(args, log):
 
 def _profile_run_gist(args, log):
     """--profile-run --workload gist1m [--n N]: the GIST-shaped batched form
-    (BF16 rows, each query with its own p, k and ef) on the block-per-query
-    kernel with the default visited table, three warm-up searches and --steps
+    (BF16 rows, each query with its own p, k and ef) on the cooperative
+    (block-per-query) kernel, three warm-up searches and --steps
     searches, L2 flushed before each.  Each search launches the two
     queue-ordering kernels, then one search launch per beam bucket (<= 64,
     128, 256, 512), largest first."""

@@ -153,10 +153,10 @@ typedef struct {
                             finished blocks leave. */
   int32_t use_graph;     /* 1: capture the launch sequence once per call shape, then replay */
   int32_t ef_max;        /* bound on ef' over the batch when per-query ef is given; 0 => 512 */
-  int32_t query_threads; /* 32 = one warp per query (4 queries per block), 128 = one block per
+  int32_t query_threads; /* 32 = one warp per query (2 queries per block), 128 = one block per
                             query (2, 4 or 8 warps sum its rows and one keeps its beam: the
                             most with which all queries of the launch are resident at once,
-                            else 2); a launch that does not fit in shared memory fails with
+                            else 4 for wide rows and 2 for others); a launch that does not fit in shared memory fails with
                             UHNSW_ECAPACITY.  0 => the configuration uhnsw_autotune chose for
                             this beam / k bucket; else, with team_lanes and stage_bytes 0 too,
                             a block per query where all queries are resident at once and for

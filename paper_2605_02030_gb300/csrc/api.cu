@@ -661,8 +661,10 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
   //   but FP32 rows that leave a fifth of a team's 128 chunks empty (300 and 400
   //     dimensions): 0.77 and 0.82 at 10,000 queries of ef 64, 1.03 to 1.25 at ef 128
   //     and 300 and, at ef 64, with 1,300 queries;
-  //   33 to 64 chunks (500 FP16, 200 and 500 FP32): 1.04 to 2.4 at ef 300;
-  //     at ef 52 and 64, 1.15 to 1.75 up to 2,500 queries, 0.67 to 1.28 above;
+  //   33 to 64 chunks (500 FP16, 200 and 250 FP32): 1.04 to 2.4 at ef 300; up to
+  //     3,000 queries at ef 52 to 100, 0.82 to 1.75.  With more queries it depends on
+  //     the rows: GIST-shaped ones 0.92 to 1.38 at ef 64 to 128 and 0.98 to 1.57 at
+  //     ef 160 and 220, a mixture of 16 clusters 0.71 to 1.03 and 0.81 to 1.04;
   //   narrower rows: 0.7 to 1.4 at 1,500 queries, 0.6 to 0.9 at 10,000.
   auto coop_anyway = [&](const WarpShape& sh, int bound) -> int {
     const int row = sh.team * sh.cpl;
@@ -975,7 +977,7 @@ extern "C" int uhnsw_verify(uhnsw_index* idx, const float* q, const float* p, co
   a.kappa = opts.kappa;
   a.tau = opts.tau != 0.f ? opts.tau : 0.92f;
   a.mode = opts.verify_mode;
-  // two tests in 128 dimensions: 5,003 queries x 300 candidates take 199 us, 208 with
+  // two tests in 128 dimensions: 5,003 queries x 300 candidates take 165 us, 177 with
   // a test after every group
   a.vgroups = opts.verify_groups > 0 ? opts.verify_groups : 3;
   a.cmax = kBlock / 8;
@@ -1098,8 +1100,8 @@ extern "C" int uhnsw_plan_t(const int32_t* counts, const float* p, int64_t n, in
   return UHNSW_OK;
 }
 
-// Scratch of uhnsw_exact_static: the per-slice partial top-k lists (distances
-// then ids) of one call.  Host code must not take this name's address (it is a
+// Scratch of uhnsw_exact_static: the per-slice top-k lists (8-byte keys) of one
+// call.  Host code must not take this name's address (it is a
 // host-side stand-in); it uses the device address looked up per device below.
 static __device__ __align__(256) unsigned char g_exact_static_scratch[UHNSW_EXACT_STATIC_BYTES];
 

@@ -27,7 +27,11 @@ cudaError_t launch_verify_warps(const QueryArgs& a, cudaStream_t st) {
 // steps of one query are then what takes the time.  Past that, two for up to
 // 256 candidates between two barriers of Algorithm 1 (the exact mode has
 // none): more warps find few rows to sum.  Two as well for up to 64 short
-// rows: in steps of 32 or 64 none of them would be dropped.
+// rows: in steps of 32 or 64 none of them would be dropped.  Around the line, two
+// and four warps, exact mode, 128 dimensions: 3,000 queries x 200 81 and 83 us, 256
+// 95 and 94, 300 108 and 108, 512 171 and 165; 8,000 x 200 197 and 190.  From 457
+// queries to about a thousand four are faster on both sides of it (600 x 200: 32 and
+// 23; 960 dimensions 163 and 102).
 cudaError_t launch_verify(const QueryArgs& a, int num_sms, cudaStream_t st) {
   if (a.cand_t <= 64 && a.d_pad <= 256) return launch_verify_warps<2>(a, st);
   if (a.nq <= 3 * (int64_t)num_sms) return launch_verify_warps<8>(a, st);
@@ -183,9 +187,10 @@ bool pick_warp_shape(uhnsw_dtype dt, int chunks, int team_pref, bool few, WarpSh
   // on two streams) two rows per team and round measured 8 % faster than
   // three (1.37 vs 1.49 ms per batch) and one row 6 % slower.  A batch too
   // small to fill the GPU's warps (`few`) is bound by each query's own
-  // latency: there three rows per round keep more loads in flight (serving
-  // batches of 7 to 33 queries: p50 7 % and p99 up to 25 % lower than with
-  // two rows).  Rows of 12 chunks (96 FP16 dimensions) take 4 lanes x 3
+  // latency: there three rows per round keep more loads in flight (2,000 to
+  // 3,600 queries, ef 52 at width 2 and ef 128: 0.92 to 0.98 of the time with
+  // two rows; batches whose queries are all resident run the cooperative
+  // kernel, which has its own number of rows).  Rows of 12 chunks (96 FP16 dimensions) take 4 lanes x 3
   // chunks, which leaves no lane on a zeroed chunk: 3.5 % faster than
   // 8 x 2 at 10M x 96, ef 512.  The shape never changes a result.
   static const WarpShape f32[] = {{8, 1, 4},  {8, 2, 2},  {16, 2, 4}, {32, 2, 2},

@@ -17,8 +17,9 @@
 // 291 us for those 5,003 queries and 137 us for one: 38 steps each, in a grid
 // of 1.2 times the resident warps.  Now 164 us back to back (4.7 TB/s of rows;
 // 0.20 ms on a cold L2) and 43 us.
-// 64 registers (1,024 threads an SM) without spills: 56 registers spill and
-// 80 hide less latency (5,003 queries, 4 warps: 208 us, 219, 253).
+// 64 registers (1,024 threads an SM) without spills: 56 registers spill and one
+// block less per SM (68 registers) hides less latency (5,003 queries, 4 warps: 165
+// us, 178, 175).
 #pragma once
 
 #include "coop_kernels.cuh"

@@ -680,8 +680,8 @@ __device__ void warp_query(const QueryArgs& a, int64_t qi, unsigned char* ws, co
 // smaller L1 cost; FP32 rows of one or two chunks a lane gain from 32 warps at
 // 64 registers where the launch's shared memory holds that many (small beams),
 // the others run 24 at 80.  32 against 24, 1M x 128 unless stated:
-//   FP32, ef 64, 10,000 queries 2.80 vs 2.93 ms, 4,000 queries 1.44 vs 1.78;
-//     L0.5 and L1 graphs 3.31 vs 4.08; 40k x 180 2.02 vs 2.32; where 32 do not
+//   FP32, ef 64, 10,000 queries 2.82 vs 2.88 ms, 4,000 queries 1.44 vs 1.78;
+//     L0.5 and L1 graphs 3.31 vs 4.01; 40k x 180 2.02 vs 2.32; where 32 do not
 //     fit, ef 200 would take 7.50 vs 7.31 and 40k x 50 at ef 300 3.63 vs 3.38;
 //   FP16 (ef 52, width 1) 2.03 vs 1.89, BF16 2.41 vs 1.96, 1M x 96 at ef 64
 //     3.37 vs 2.85.
