@@ -618,8 +618,8 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
     for (int i = kCoopForms - 1; i >= -1; --i) {
       const int nw = i >= 0 ? kCoopWarps[i] : fallback;
       if (nw == 0) return false;
-      sh.most = i < 0 && nw == kCoopManyWarps;
       const int cmax = (std::max(width * deg0, deg) + nw - 1) / nw * nw;
+      sh.most = i < 0 && cmax <= 32 * nw;
       const int ext = sh.team * sh.cpl * (idx->tdtype == UHNSW_F32 ? 4 : 8);
       int hb = visited_bits(hash, bound, width, deg0);
       size_t smem = CoopLayout(ext, bound, hb, cmax, k_max, nw + 1).total;
@@ -645,13 +645,13 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
   };
 
   // Distance warps per query of a cooperative launch whose queries are not all
-  // resident (the measurements are at kCoopManyWarps): four for rows above 64
-  // chunks and for FP32 rows above 32, two for shorter ones (400k x 500 FP16, ef
-  // 64: 5.1 ms with two and 5.8 with four; 1M x 128 FP16 2.9 and 3.2) and for FP32
-  // rows of 16 chunks a lane (50k x 2,000: 15.6 and 16.4).
+  // resident (the measurements are at coop_has_many): four for rows above 64 chunks,
+  // two for shorter ones, for FP32 rows of four chunks a lane (200k x 500 GIST-shaped,
+  // ef 300: 16.6 and 18.5 ms with two and four; 200k x 300 of a mixture 38.9 and 34.5)
+  // and of sixteen (50k x 2,000, ef 64, before the sharing: 15.6 and 16.4).
   auto coop_warps = [&](const WarpShape& sh) -> int {
-    const int row = sh.team * sh.cpl;
-    return sh.cpl <= 8 && (row > 64 || (row > 32 && idx->tdtype == UHNSW_F32)) ? kCoopManyWarps : 2;
+    const bool two = sh.cpl > 8 || (sh.cpl == 4 && idx->tdtype == UHNSW_F32);
+    return sh.team * sh.cpl > 64 && !two ? 4 : 2;
   };
 
   // The same, where the warp kernel could take the launch (0: it does).  The
@@ -661,10 +661,11 @@ int prepare_search(uhnsw_index* idx, const float* q, const float* p, const int32
   //   but FP32 rows that leave a fifth of a team's 128 chunks empty (300 and 400
   //     dimensions): 0.77 and 0.82 at 10,000 queries of ef 64, 1.03 to 1.25 at ef 128
   //     and 300 and, at ef 64, with 1,300 queries;
-  //   33 to 64 chunks (500 FP16, 200 and 250 FP32): 1.04 to 2.4 at ef 300; up to
-  //     3,000 queries at ef 52 to 100, 0.82 to 1.75.  With more queries it depends on
-  //     the rows: GIST-shaped ones 0.92 to 1.38 at ef 64 to 128 and 0.98 to 1.57 at
-  //     ef 160 and 220, a mixture of 16 clusters 0.71 to 1.03 and 0.81 to 1.04;
+  //   33 to 64 chunks: 0.79 to 1.40 at 10,000 queries of ef 64 (200 and 250 FP32, 400
+  //     and 500 16-bit); before the warps shared a step's rows, 0.82 to 1.75 up to
+  //     3,000 queries at ef 52 to 100 and, with more, 0.71 to 1.38 at ef 64 to 128 and
+  //     0.81 to 1.57 at ef 160 and 220 (a mixture of 16 clusters the least, GIST-shaped
+  //     rows the most);
   //   narrower rows: 0.7 to 1.4 at 1,500 queries, 0.6 to 0.9 at 10,000.
   auto coop_anyway = [&](const WarpShape& sh, int bound) -> int {
     const int row = sh.team * sh.cpl;

@@ -455,7 +455,7 @@ __device__ __forceinline__ void coop_invalid(const QueryArgs& a, int64_t qi) {
   if (threadIdx.x == 0) put_stats(a, qi, 0, 0, 0, 0, 0, UHNSW_EINVAL, 0, 0);
 }
 
-template <typename T, int TEAM, int CPL, int U, int NW>
+template <typename T, int TEAM, int CPL, int U, int NW, bool MANY>
 __device__ void coop_query(const QueryArgs& a, int64_t qi, unsigned char* smem,
                            const CoopLayout& L) {
   constexpr int VEC = Elems16<T>::n;
@@ -616,6 +616,18 @@ __device__ void coop_query(const QueryArgs& a, int64_t qi, unsigned char* smem,
     }
   }
 
+  // MANY: a warp that is done with the rows of its own links, and the merge warp after
+  // its merge, takes rounds of the other warps' rows (posted: how many rows a warp
+  // has, -1 before it knows; cursor: the next one to take; [2][NW] each, by the
+  // step's parity, in the merge warp's link buffer, which has no other use).  A row's
+  // key has its place whoever sums it, so that the candidates are the same.
+  volatile int* posted = reinterpret_cast<volatile int*>(smem + L.wl) + NW * 32;
+  int* cursor = reinterpret_cast<int*>(smem + L.wl) + NW * 32 + 2 * NW;
+  if (MANY && tid < 2 * NW) {
+    posted[tid] = -1;
+    cursor[tid] = 0;
+  }
+
   // layer-0 search from W = {cur}; its first parent is cur
   if (tid == 0) {
     hash_insert(tab, hb, (int32_t)key_id(curk), a.err);
@@ -663,7 +675,46 @@ __device__ void coop_query(const QueryArgs& a, int64_t qi, unsigned char* smem,
       ++nres;
       __syncthreads();
     }
-    if (!merger) {
+    if constexpr (MANY) {
+      unsigned long long* out = ckbuf(ph ^ 1);
+      const int at = (ph ^ 1) * NW;
+      if (!merger) {
+        const bool in = lane < spw && slot < npar * g.deg0;
+        const int j = in ? slot / g.deg0 : 0;
+        const uint32_t mine = __shfl_sync(kFull, par, j);
+        const int32_t v =
+            in ? g.ell0[chk_idx(mine, a.n, 5, a.err) * g.deg0 + (slot - j * g.deg0)] : -1;
+        const bool fresh = v >= 0 && hash_insert(tab, hb, v, a.err);
+        const unsigned mask = __ballot_sync(kFull, fresh);
+        const int nf = __popc(mask);
+        if (fresh) wl[__popc(mask & lanemask_lt())] = (uint32_t)chk_idx(v, a.n, 1, a.err);
+        if (lane >= nf && lane < spw) out[warp * spw + lane] = kNoKey;
+        __syncwarp();
+        if (lane == 0) {
+          fresh_of[at + warp] = nf;
+          posted[ph * NW + warp] = -1;  // (the next step's)
+          cursor[ph * NW + warp] = 0;
+          __threadfence_block();
+          posted[at + warp] = nf;
+        }
+        __syncwarp();
+      }
+      for (int i = 0; i < NW; ++i) {
+        const int w = (warp + i) % NW;
+        int n = lane == 0 ? posted[at + w] : 0;
+        n = __shfl_sync(kFull, n, 0);
+        __threadfence_block();
+        const uint32_t* ids = reinterpret_cast<const uint32_t*>(smem + L.wl) + w * 32;
+        constexpr int kRound = U * (32 / TEAM);
+        while (n > 0) {
+          int c = lane == 0 ? atomicAdd(&cursor[at + w], kRound) : 0;
+          c = __shfl_sync(kFull, c, 0);
+          if (c >= n) break;
+          coop_dist_metric<T, TEAM, CPL, U, QREG>(rt.metric, rt.bp, trav, a.d_pad, qs, qv, ids + c,
+                                                  min(kRound, n - c), out + w * spw + c);
+        }
+      }
+    } else if (!merger) {
       unsigned long long* out = ckbuf(ph ^ 1);
       int nf = 0;
       if (ahead) {
@@ -800,33 +851,35 @@ struct CoopMinBlocks {
                                           : 3;
 };
 
-// The form for more queries than are resident, of rows whose sums are what a step
-// takes: four distance warps and a block more per SM.  A resident query is slower
-// in it (300 to 600 queries of 1M x 128 and 400k x 500 FP16, ef 64: 1.05 to 1.18
-// times the time), so that those keep CoopMinBlocks.  10,000 queries, ms; this
-// form, two distance warps, and the kernel they replaced (four warps per query, each
-// summing and merging in turn):
-//   1M x 960 BF16, ef 512, k 100                          90.4, 108.5, 101.5
-//   the same rows, mixed k and ef, one launch             37.4, 44.8, 48.2
-//   the same, launches queued on two streams              38.3, 45.8, 37.9
-//   200k x 960 FP16, ef 64 and 300                        6.5, 7.7, 10.8; 19.5, 20.0, 37.4
-//   200k x 960 FP32                                       11.3, 16.1, 14.6; 27.9, 36.0, 45.5
-//   200k x 200 FP32                                       4.1, 4.4, 3.6; 19.9, 21.9, 17.9
-// Four warps at CoopMinBlocks' four blocks took 100.9 ms for the first row, eight
-// 129.8; two warps at seven blocks 118.8.  FP32 rows of four chunks a lane would
-// spill at five blocks and take four warps at four (200k x 400, ef 64: 5.9 ms, 6.3
-// with spills, 6.8 with two warps).
-constexpr int kCoopManyWarps = 4;
-template <typename T, int TEAM, int CPL>
+// The form for more queries than are resident (MANY), for rows whose sums are what
+// a step takes: the warps of a block share a step's rows.  A link is fresh or not by
+// chance, and a distance warp that finds few fresh ones, or the merge warp once it has
+// merged, waited for the slowest (the barrier was 7.7 of the 17.7 cycles between two
+// instructions of a warp at 200k x 200 FP32).  Two distance warps for rows of two chunks a lane and FP32 rows of four, four
+// for longer ones (coop_warps in the host code).  10,000 queries, ms: this form;
+// without the sharing; two distance warps without it; and the kernel before the
+// cooperative one (four warps per query, each summing and merging in turn):
+//   1M x 960 BF16, ef 512, k 100                         75.5, 107, 129, 103
+//   the same rows, mixed k and ef, one launch            31.1, 43.9, 52.8, 52.8
+//   the same, launches queued on two streams             31.9, 45.1, 54.0, 41.2
+//   200k x 960 FP16, ef 64 and 300                       6.6, 6.6, 7.8, 10.8; 20.6, 19.6, 20.3, 37.4
+//   100k x 800 FP32, ef 64 and 300                       11.4, 13.8, 20.7; 34.8, 43.1, 60.2
+//   200k x 200 FP32, ef 64 and 300                       3.7, 4.2, 4.4, 3.6; 17.3, 19.9, 21.6, 17.9
+// A block per SM more than CoopMinBlocks asks (72 registers) for 16-bit rows of four
+// chunks: with four blocks the first row takes 83.5 ms.  Resident queries keep the
+// registers of CoopMinBlocks (300 to 600 queries took 1.05 to 1.18 times as long).
+template <typename T, int TEAM, int CPL, int NW>
 constexpr bool coop_has_many() {
-  return TEAM == 32 && (CPL == 8 || CPL == (std::is_same<T, float>::value ? 2 : 4));
+  constexpr bool f32 = std::is_same<T, float>::value;
+  return TEAM == 32 &&
+         (NW == 4 ? CPL == 8 || (CPL == 4 && !f32) : NW == 2 && (CPL == 2 || (CPL == 4 && f32)));
 }
-template <int CPL>
-constexpr int kCoopManyBlocks = CPL <= 4 ? 5 : 4;
+template <int CPL, int NW, bool MANY>
+constexpr int kCoopBlocks = !MANY || NW == 2 ? CoopMinBlocks<CPL, NW>::value : CPL == 4 ? 5 : 4;
 
 // One block of NW + 1 warps per query; a.queue_head set = persistent.
-template <typename T, int TEAM, int CPL, int U, int NW, int BLOCKS>
-__global__ void __launch_bounds__((NW + 1) * 32, BLOCKS)
+template <typename T, int TEAM, int CPL, int U, int NW, bool MANY>
+__global__ void __launch_bounds__((NW + 1) * 32, (kCoopBlocks<CPL, NW, MANY>))
     uhnsw_csearch_kernel(const QueryArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int next;
@@ -845,7 +898,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, BLOCKS)
       qi = next;
     }
     if (qi >= a.nq) break;
-    coop_query<T, TEAM, CPL, U, NW>(a, qi, smem, L);
+    coop_query<T, TEAM, CPL, U, NW, MANY>(a, qi, smem, L);
     __syncthreads();
     if (!a.queue_head) break;
   }

@@ -19,9 +19,9 @@ struct CoopRows {
 template <typename T, int TEAM, int CPL, int NW>
 auto csearch_kernel(bool most) {
   constexpr int U = CoopRows<CPL>::value;
-  auto kern = uhnsw_csearch_kernel<T, TEAM, CPL, U, NW, CoopMinBlocks<CPL, NW>::value>;
-  if constexpr (NW == kCoopManyWarps && coop_has_many<T, TEAM, CPL>())
-    if (most) kern = uhnsw_csearch_kernel<T, TEAM, CPL, U, NW, kCoopManyBlocks<CPL>>;
+  auto kern = uhnsw_csearch_kernel<T, TEAM, CPL, U, NW, false>;
+  if constexpr (coop_has_many<T, TEAM, CPL, NW>())
+    if (most) kern = uhnsw_csearch_kernel<T, TEAM, CPL, U, NW, true>;
   return kern;
 }
 

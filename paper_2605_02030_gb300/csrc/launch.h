@@ -14,8 +14,8 @@ namespace uhnsw_dev {
 // U rows per team loaded per round; kWarpsPerBlock warps (queries) per block.
 struct WarpShape {
   int team, cpl, u;
-  bool most = false;  // the form with more queries per SM (warp kernel: 32, not 24;
-                      // cooperative kernel: kCoopManyWarps distance warps)
+  bool most = false;  // warp kernel: the form for 32 warps per SM, not 24; cooperative
+                      // kernel: the form for more queries than are resident
 };
 constexpr int kWarpsPerBlock = 2;
 // The warp kernel's team shape for rows of `chunks` 16-byte chunks.
