@@ -221,8 +221,10 @@ __device__ __forceinline__ float root_p(float s, float p) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rden) : "f"((float)den));
   const double rd = (double)rden;
   double u = num * rd;
-  u = fma(fma(-u, den, num), rd, u);  // 2^-46
-  u = fma(fma(-u, den, num), rd, u);  // as far as FP64 goes
+  // 2^-46, then as far as FP64 goes (as a loop: unrolled, the step moves registers in
+  // the search kernels, and 1,000 queries of 1M x 96 FP16 at ef 512 take 1 % longer)
+#pragma unroll 1
+  for (int i = 0; i < 2; ++i) u = fma(fma(-u, den, num), rd, u);
   const double w = u * u;
   const float wf = (float)w;
   float lt = fmaf(wf, 1.0f / 19, 1.0f / 17);
